@@ -174,6 +174,13 @@ namespace escg_impl {
 // 2^32), q = round(p 2^32) -- exact integer arithmetic, so the value does not
 // depend on the compiler's floating-point contraction; prob == nullptr
 // means every edge is certain (T_XI).
+bool edges_certain(int S, const uint8_t* D, const double* prob) {
+  if (!prob) return true;
+  for (int k = 0; k < S * S; ++k)
+    if (D[k] && prob[k] < 1.0) return false;
+  return true;
+}
+
 void build_transitions(int S, const uint8_t* D, const double* prob, uint64_t tx, uint64_t txi,
                        uint32_t* out) {
   const int s1 = S + 1;
@@ -812,6 +819,7 @@ escg_t* escg_create_ex(int32_t L, int32_t S, const uint8_t* digraph, const escg_
   d.tx = tx >> 32 ? 0xFFFFFFFFu : (uint32_t)tx;
   d.txi = txi >> 32 ? 0xFFFFFFFFu : (uint32_t)txi;
   d.S = S;
+  d.certain = edges_certain(S, digraph, o.dominance_prob) ? 1 : 0;
   fill_perm24(d.perm24);
   bool uni = true;
   for (int k = 0; k < p.P; ++k) uni = uni && (p.cs[k + 1] - p.cs[k] == 64);

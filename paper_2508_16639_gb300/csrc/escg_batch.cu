@@ -1125,6 +1125,7 @@ int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int s
   d.txi = txi >> 32 ? 0xFFFFFFFFu : (uint32_t)txi;
   d.S = sp.S;
   d.uniform64 = 0;
+  d.certain = edges_certain(sp.S, sp.digraph, sp.dominance_prob) ? 1 : 0;
   fill_perm24(d.perm24);
   sd.done = reinterpret_cast<uint32_t*>(base + pl.done);
   sd.max_mcs = (uint32_t)sp.max_mcs;

@@ -45,6 +45,9 @@ void set_last_error(const char* fmt, ...);
 void build_transitions(int S, const uint8_t* D, const double* prob, uint64_t tx, uint64_t txi,
                        uint32_t* out);
 
+// Whether every edge of the digraph D has probability 1 (prob as above).
+bool edges_certain(int S, const uint8_t* D, const double* prob);
+
 // Host-side launchers (all asynchronous on `stream`).
 cudaError_t launch_init(const LatticeDesc& d, uint64_t T_empty, cudaStream_t stream);
 // Packed lattice (d.bits 4 or 2) from / to a byte image of byte_pitch-byte rows.

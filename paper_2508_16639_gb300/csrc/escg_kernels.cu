@@ -22,6 +22,7 @@
 
 #include "escg_device.cuh"
 #include "escg_resident.cuh"
+#include "escg_resident_patch.cuh"
 #include "escg_rule8.cuh"
 #include "escg_internal.h"
 #include "escg_tma.cuh"
@@ -1599,6 +1600,46 @@ __global__ void __launch_bounds__(kResThreads) resident_kernel(PersistentArgs a)
   if (threadIdx.x == 0 && !st->stopped) st->mcs = m_end;
 }
 
+// The same on the macro layout (escg_resident_patch.cuh).  Bound by the chain
+// of sixteen fine phases an MCS.  Measured against the one-byte image, us per
+// MCS: L = 64 (S = 3, no movement) 17.7 -> 5.8, 64 18.4 -> 5.7, 100 (S = 5) 32.2
+// -> 16.9, 160 25.7 -> 17.7, 191 (S = 5) 35.9 -> 30.6; on request L = 256 41.6 ->
+// 32.8, 400 142 -> 83.  640 threads keep 96 registers a thread; a phase of L =
+// 64 has 64 sub-blocks, so eight groups of 64 threads take the phases in turn.
+constexpr int kResPatchThreads = 640;
+template <int PL, int LG, bool REFLECT>
+__global__ void __launch_bounds__(kResPatchThreads, 1) resident_patch_kernel(const __grid_constant__ PersistentArgs a,
+                                                                            int gs) {
+  extern __shared__ __align__(16) uint8_t res_dyn[];
+  __shared__ ResidentPatchSmem S;
+  const LatticeDesc& d = a.d;
+  RunState* st = a.st;
+  if (ld_volatile(&st->stopped)) return;
+  const ResidentLayout R = resident_layout(d, PL);
+  resident_setup<PL>(d, R, res_dyn, S);
+  __syncthreads();
+  resident_fill<PL>(d, R, res_dyn);
+  const uint32_t m_end = a.m_begin + a.n_mcs;
+  resident_run_patch<PL, LG, REFLECT>(d, R, res_dyn, S, gs, a.m_begin, m_end, a.log_every,
+                                      [&](uint32_t mm, const uint32_t* hist) {
+    unsigned long long c[kMaxStates];
+    for (int v = 0; v < kMaxStates; ++v) c[v] = v <= d.S ? hist[v] : 0u;
+    write_log_entry(st, a.lb, d.S, mm, a.log_every, c, a.stop_at_extinction);
+    return st->stopped != 0u;
+  });
+  resident_drain<PL>(d, R, res_dyn);
+  if (threadIdx.x == 0 && !st->stopped) st->mcs = m_end;
+}
+
+static const void* resident_patch_fn(const LatticeDesc& d) {
+  const bool one = patch_planes(d) == 1, moore = d.nbh == 8, refl = d.reflect != 0;
+#define RES_FN(PL, LG, RF) reinterpret_cast<const void*>(&resident_patch_kernel<PL, LG, RF>)
+  if (one)
+    return moore ? (refl ? RES_FN(1, 3, true) : RES_FN(1, 3, false)) : (refl ? RES_FN(1, 2, true) : RES_FN(1, 2, false));
+  return moore ? (refl ? RES_FN(2, 3, true) : RES_FN(2, 3, false)) : (refl ? RES_FN(2, 2, true) : RES_FN(2, 2, false));
+#undef RES_FN
+}
+
 // Largest dynamic shared memory a resident launch may use on this device.
 int resident_max_dyn_bytes(int device) {
   int optin = 0;
@@ -1610,7 +1651,21 @@ bool resident_fits(const LatticeDesc& d, int device) {
   return d.P <= 8 && d.Py <= 8 && resident_dyn_bytes(d.L, d.H) <= resident_max_dyn_bytes(device);
 }
 
+// Partitions with a 4-site segment (sides of 13 to 15 sites) run on the
+// one-byte image; every other lattice that fits runs on macros, whose image
+// is at most half as large.
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream) {
+  if (slot_axis_ok(a.d.ax) && slot_axis_ok(a.d.ay)) {
+    const int bytes = resident_layout(a.d, patch_planes(a.d)).bytes;
+    const void* fn = resident_patch_fn(a.d);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    int gs = 0, nt = 0;
+    resident_threads(a.d, kResPatchThreads, &gs, &nt);
+    PersistentArgs args = a;
+    void* params[] = {&args, &gs};
+    return cudaLaunchKernel(fn, dim3(1), dim3(nt), params, (size_t)bytes, stream);
+  }
   const int bytes = resident_dyn_bytes(a.d.L, a.d.H);
   cudaError_t e = cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;

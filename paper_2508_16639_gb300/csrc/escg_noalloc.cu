@@ -175,6 +175,7 @@ extern "C" int escg_run_noalloc(uint8_t* d_lattice, int32_t L, int32_t S, const 
   d.nbh = 4;
   d.reflect = 0;
   d.uniform64 = (L % 64 == 0 && L / 64 == P && d.pitch % 16 == 0) ? 1 : 0;
+  d.certain = 1;
   fill_perm24(d.perm24);
 
   NoallocSetup su;

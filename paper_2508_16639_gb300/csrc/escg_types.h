@@ -111,6 +111,9 @@ struct LatticeDesc {
   int32_t uniform_var;  // all blocks 64x64 with 2x2 sub-blocks, one byte per site,
                         // and a rule variant (Moore and/or reflecting): the flag
                         // kernel's uniform variant visit
+  int32_t certain;      // every dominance edge certain (no pair's interaction
+                        // threshold below txi): with S <= 3 a step's rule fits
+                        // a 64-bit word (escg_patch.cuh)
 };
 
 // Fills perm24 with the 24 orders of the colours {0,1,2,3} in lexicographic
