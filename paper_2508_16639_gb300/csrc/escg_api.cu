@@ -260,6 +260,8 @@ struct escg {
   int own_dyn = 0;               // its shared-memory padding
   int own_threads = 0;           // and CTA size
   int flag_threads = 256;        // CTA size of the flag kernel (128: uniform geometry, > 4 CTAs per SM)
+  bool use_macro = false;        // flag kernel on macros (uniform geometry)
+  void* d_macros = nullptr;      // its macro array, kept for the handle's life
   bool use_gown = false;         // block owners on a generic partition
   int tuned_mode = 0, tuned_ctas = 0;   // autotuner's choice (launch mode, CTAs per SM)
   double tuned_ms_per_mcs = 0.0;
@@ -413,6 +415,7 @@ void free_handle(escg* h) {
   cudaFree(h->d_log_mcs);
   cudaFree(h->d_done);
   cudaFree(h->d_ob);
+  cudaFree(h->d_macros);
   cudaFree(h->d_scratch);
   for (auto& e : h->ev_used) {
     cudaEventDestroy(e.first);
@@ -440,6 +443,17 @@ int ensure_records(escg* h, size_t words) {
   return ESCG_OK;
 }
 
+// The macro array of the flag kernel, a quarter of the one-byte lattice (half
+// with 4 bits per site), allocated on first use; false if there is no room
+// (the flag kernel then works on the lattice array itself).
+bool ensure_macros(escg* h) {
+  if (h->d_macros) return true;
+  if (cudaMalloc(&h->d_macros, macro_bytes(h->desc)) == cudaSuccess) return true;
+  cudaGetLastError();
+  h->d_macros = nullptr;
+  return false;
+}
+
 // Picks the lattice-update kernel for launch mode `persistent` (escg_options)
 // and the CTAs per SM of the ticketed kernels (0: as many as fit), from the
 // partition, the storage and the device's occupancy.  Physical mapping only:
@@ -452,7 +466,8 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   h->use_tma = h->use_ll = h->use_own = h->use_gown = h->use_resident = false;
   h->own_dyn = h->own_threads = 0;
   h->gown = GownConfig{};
-  h->grid = persistent_grid(h->device, d.uniform64 != 0 || d.uniform_var != 0);
+  h->use_macro = false;
+  h->grid = persistent_grid(h->device, d.uniform64 != 0 && h->bits == 8);
   // the TMA and mailbox kernels are written for square lattices of one byte
   // per site; the flag kernel takes rectangular and packed ones in both
   // geometries
@@ -531,10 +546,14 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   // several waves deep and throughput, not the colour chain, binds.
   h->flag_threads = 256;
   const bool flag = !h->use_tma && !h->use_ll && !h->use_own && !h->use_gown && !h->use_resident;
-  const bool deep = persistent == 1 && (int64_t)p.P * py.P / 4 >= (int64_t)kFlag128Ratio * h->grid;
-  if (flag && (ctas_per_sm > 4 || deep) && d.uniform64) {
-    h->flag_threads = 128;
-    h->grid = persistent_grid128(h->device);
+  if (flag && persistent != 0 && d.blocks64 && ensure_macros(h)) {
+    h->use_macro = true;
+    h->grid = persistent_macro_grid(d, h->device, 256);
+    const bool deep = persistent == 1 && (int64_t)p.P * py.P / 4 >= (int64_t)kFlag128Ratio * h->grid;
+    if (ctas_per_sm > 4 || deep) {
+      h->flag_threads = 128;
+      h->grid = persistent_macro_grid(d, h->device, 128);
+    }
   }
   if (ctas_per_sm > 0) {
     int sms = 0;
@@ -828,10 +847,10 @@ escg_t* escg_create_ex(int32_t L, int32_t S, const uint8_t* digraph, const escg_
   for (int k = 0; k < py.GQ; ++k) uni = uni && (py.fs[k + 1] - py.fs[k] == 2);
   d.nbh = o.neighbourhood;
   d.reflect = o.reflecting_boundary;
-  // the uniform kernels implement the von Neumann, periodic rule; the flag
-  // kernel also the variants on 64 x 64 blocks of one byte per site
-  d.uniform64 = (uni && h->pitch % 16 == 0 && d.nbh == 4 && !d.reflect) ? 1 : 0;
-  d.uniform_var = (uni && h->pitch % 16 == 0 && (d.nbh == 8 || d.reflect) && h->bits == 8) ? 1 : 0;
+  // the owner, mailbox and TMA kernels of the uniform geometry implement the
+  // von Neumann, periodic rule, the flag kernel on macros every rule
+  d.blocks64 = (uni && h->pitch % 16 == 0) ? 1 : 0;
+  d.uniform64 = (d.blocks64 && d.nbh == 4 && !d.reflect) ? 1 : 0;
   if (select_kernel(h, o.persistent, o.ctas_per_sm) != ESCG_OK) return fail(ESCG_ENOMEM);
 
   if (launch_init(d, h->T_empty, h->stream) != cudaSuccess) {
@@ -864,8 +883,8 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
   }
   const uint32_t k = h->opt.log_every;
   // rule variants count log points with the count kernel between launches
-  // (the resident kernel counts in-kernel for every rule)
-  const bool fused = (h->desc.nbh == 4 && !h->desc.reflect) || h->use_resident;
+  // (the resident kernel and the one on macros count in-kernel for every rule)
+  const bool fused = (h->desc.nbh == 4 && !h->desc.reflect) || h->use_resident || h->use_macro;
   while (h->mcs_enq < target) {
     uint64_t end;
     if (h->opt.persistent && !h->opt.stop_at_extinction && fused) {
@@ -913,6 +932,10 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
         CUDA_TRY(launch_persistent_tma(ta, grid, h->stream));
       } else if (h->use_ll) {
         CUDA_TRY(launch_persistent_ll(a, grid, h->stream));
+      } else if (h->use_macro) {
+        a.macros = h->d_macros;
+        CUDA_TRY(launch_persistent_macro(a, grid, h->stream));
+        h->launches += 2;   // the array into macros and back
       } else {
         CUDA_TRY(launch_persistent(a, grid, h->stream));
       }

@@ -86,8 +86,9 @@ struct PersistentArgs {
   int32_t stall_block;   // test hook: never publish this block's epoch (-1: off)
   unsigned long long* ob;  // boundary records of the mailbox kernel ([P*P][4][32]), else null
   int32_t fuse_counts;     // 1: counts of log points fused into the visits; 0: the host counts
-  int32_t threads;         // flag kernel on uniform one-byte lattices: 128 (two quads per
-                           // thread, up to 8 CTAs per SM) or 0 / 256 (one quad per thread)
+  int32_t threads;         // flag kernel on macros: 128 (two sub-blocks per thread, up to 8
+                           // CTAs per SM) or 256 (one)
+  void* macros;            // macro array of the flag kernel on uniform partitions (escg_flag.cu)
   // div_rcp32 of the ticket decode's divisors (blocks per MCS, blocks per
   // coarse phase, half the blocks per row); filled in by launch_persistent
   uint32_t rcp_nb, rcp_per, rcp_half;
@@ -97,8 +98,12 @@ struct PersistentArgs {
 cudaError_t launch_persistent(const PersistentArgs& a, int grid, cudaStream_t stream);
 // Occupancy-derived grid size of the persistent kernel for a lattice.
 int persistent_grid(int device, bool uniform);
-// The same for the 128-thread build of the uniform flag kernel (up to 8 per SM).
-int persistent_grid128(int device);
+// The flag kernel on macros (uniform partitions, any rule; escg_flag.cu): the
+// lattice array is turned into a.macros (macro_bytes), run there by CTAs of
+// a.threads and written back.  Grid by occupancy.
+size_t macro_bytes(const LatticeDesc& d);
+int persistent_macro_grid(const LatticeDesc& d, int device, int threads);
+cudaError_t launch_persistent_macro(const PersistentArgs& a, int grid, cudaStream_t stream);
 
 // Whole-lattice residency: one CTA runs MCS [m_begin, m_begin + n_mcs) with
 // the lattice in shared memory (counts of log points written in-kernel).

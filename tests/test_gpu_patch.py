@@ -49,3 +49,24 @@ def test_resident_edge_probabilities(S, K):
     prob = np.zeros((S, S))
     prob[D] = np.linspace(0.0, 1.0, int(D.sum()))
     _check("resident_kernel", 67, 90, S, K, 0.5, 17, prob=prob, persistent=4)
+
+
+@pytest.mark.parametrize("L,H", [(128, 128), (256, 128), (384, 640)])
+@pytest.mark.parametrize("bits,S,K,X", [(8, 3, (1,), 1e6), (8, 15, (1, 2, 3), 0.0), (4, 5, (1, 2), 3.0),
+                                        (2, 3, (1,), 40.0)])
+def test_flag_kernel_macros(L, H, bits, S, K, X):
+    """Both CTA sizes (more than 4 CTAs per SM: 128 threads)."""
+    for ctas in (0, 8):
+        _check("persistent_kernel", L, H, S, K, X, L + 3 * H + S, persistent=3, bits_per_site=bits, ctas_per_sm=ctas)
+
+
+@pytest.mark.parametrize("nbh,reflect", [(8, False), (4, True), (8, True)], ids=["moore", "reflect", "both"])
+@pytest.mark.parametrize("bits,S,K", [(8, 3, (1,)), (8, 5, (1, 2)), (2, 3, (1,)), (4, 5, (1, 2))])
+def test_flag_kernel_macros_variants(nbh, reflect, bits, S, K):
+    _check("persistent_kernel", 256, 384, S, K, 5.0, 77 + nbh + bits, persistent=3, neighbourhood=nbh,
+           reflecting_boundary=reflect, bits_per_site=bits)
+
+
+def test_flag_kernel_macros_edge_probabilities():
+    prob = np.where(O.circulant(3, (1,)) > 0, 0.4, 0.0)
+    _check("persistent_kernel", 256, 256, 3, (1,), 1.0, 5, prob=prob, persistent=3)
