@@ -40,14 +40,23 @@ __host__ __device__ __forceinline__ uint4 philox10(uint4 c, uint32_t k0, uint32_
 // Same, with the ten round keys precomputed (rk[2r], rk[2r+1] = key + r *
 // Weyl constants); rk points into the kernel's parameter space, so the keys
 // are constant-bank operands of the XORs rather than per-thread additions.
-__device__ __forceinline__ uint4 philox10_rk(uint4 c, const uint32_t* __restrict__ rk) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint64_t p0 = (uint64_t)0xD2511F53u * c.x;
-    const uint64_t p1 = (uint64_t)0xCD9E8D57u * c.z;
-    c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ rk[2 * r], (uint32_t)p1,
-                   (uint32_t)(p0 >> 32) ^ c.w ^ rk[2 * r + 1], (uint32_t)p0);
+// AddKeys stands in for rk where the key is not a kernel parameter (the batch
+// engine): twenty keys from shared memory would take as many registers.
+struct AddKeys {
+  uint32_t k0, k1;
+  __host__ __device__ __forceinline__ uint32_t operator[](int i) const {
+    return (i & 1) ? k1 + (uint32_t)(i >> 1) * 0xBB67AE85u : k0 + (uint32_t)(i >> 1) * 0x9E3779B9u;
   }
+};
+__device__ __forceinline__ uint4 philox_round(uint4 c, uint32_t k0, uint32_t k1) {
+  const uint64_t p0 = (uint64_t)0xD2511F53u * c.x;
+  const uint64_t p1 = (uint64_t)0xCD9E8D57u * c.z;
+  return make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1, (uint32_t)p0);
+}
+template <class RK>
+__device__ __forceinline__ uint4 philox10_rk(uint4 c, RK rk) {
+#pragma unroll
+  for (int r = 0; r < 10; ++r) c = philox_round(c, rk[2 * r], rk[2 * r + 1]);
   return c;
 }
 

@@ -1577,7 +1577,7 @@ __global__ void __launch_bounds__(kResPatchThreads, 1) resident_patch_kernel(con
   __syncthreads();
   resident_fill<PL>(d, R, res_dyn);
   const uint32_t m_end = a.m_begin + a.n_mcs;
-  resident_run_patch<PL, LG, REFLECT>(d, R, res_dyn, S, gs, a.m_begin, m_end, a.log_every,
+  resident_run_patch<PL, LG, REFLECT>(d, d.rk, R, res_dyn, S, gs, blockDim.x, a.m_begin, m_end, a.log_every,
                                       [&](uint32_t mm, const uint32_t* hist) {
     unsigned long long c[kMaxStates];
     for (int v = 0; v < kMaxStates; ++v) c[v] = v <= d.S ? hist[v] : 0u;

@@ -108,10 +108,27 @@ __device__ __forceinline__ uint32_t patch_delta(const LatticeDesc& d, uint32_t a
   return (a ^ (n & 15u)) | ((b ^ (n >> 4)) << 4);
 }
 
-// Fills the tables; threads t0, t0 + n, ... of the caller.
+// Entries of the rule tables.
+__device__ __forceinline__ uint2 patch_act_entry(const LatticeDesc& d, uint32_t act) {
+  uint64_t f = 0;
+  for (int b = 0; b <= d.S; ++b)
+    for (int a = 0; a <= d.S; ++a) {
+      if (a == b) continue;
+      const uint32_t x = patch_delta(d, (uint32_t)a, (uint32_t)b, act);
+      f |= (uint64_t)((x & 3u) | (((x >> 4) & 3u) << 2)) << (4 * (4 * b + a) + 2);
+    }
+  return make_uint2((uint32_t)f, (uint32_t)(f >> 32));
+}
+__device__ __forceinline__ uint2 patch_rule_entry(const LatticeDesc& d, uint32_t a, uint32_t b) {
+  uint32_t x = 0;
+  for (uint32_t c = 0; c < 3u; ++c) x |= patch_delta(d, a, b, c) << (8u * c);
+  return make_uint2(x, reinterpret_cast<const uint32_t*>(d.trans)[kTransPairs + a * (uint32_t)(d.S + 1) + b]);
+}
+
+// Fills the tables of the geometry, then all; threads t0, t0 + n, ... of the
+// caller.
 template <int PL>
-__device__ __forceinline__ void patch_tables_fill(PatchTables& T, const LatticeDesc& d, int t0, int n) {
-  const int nbh = d.nbh == 8 ? 8 : 4, S1 = d.S + 1;
+__device__ __forceinline__ void patch_tables_geometry(PatchTables& T, int nbh, int t0, int n) {
   for (int e = t0; e < 4 * nbh; e += n) {
     const uint2 p = patch_pair(e, 2, 2, nbh);
     if (PL == 1) {
@@ -126,24 +143,17 @@ __device__ __forceinline__ void patch_tables_fill(PatchTables& T, const LatticeD
                                 : (e < 12 * nbh ? patch_pair(e - 6 * nbh, 2, 3, nbh) : patch_pair(e - 12 * nbh, 3, 3, nbh));
     T.irr[e] = make_uint2((uint32_t)PL * p.x, (uint32_t)PL * p.y);
   }
+}
+template <int PL>
+__device__ __forceinline__ void patch_tables_fill(PatchTables& T, const LatticeDesc& d, int t0, int n) {
+  patch_tables_geometry<PL>(T, d.nbh == 8 ? 8 : 4, t0, n);
+  const int S1 = d.S + 1;
   if (PL == 1) {
-    for (int k = t0; k < 3; k += n) {
-      uint64_t f = 0;
-      for (int b = 0; b < S1; ++b)
-        for (int a = 0; a < S1; ++a) {
-          if (a == b) continue;
-          const uint32_t x = patch_delta(d, (uint32_t)a, (uint32_t)b, (uint32_t)k);
-          f |= (uint64_t)((x & 3u) | (((x >> 4) & 3u) << 2)) << (4 * (4 * b + a) + 2);
-        }
-      T.act[k] = make_uint2((uint32_t)f, (uint32_t)(f >> 32));
-    }
+    for (int k = t0; k < 3; k += n) T.act[k] = patch_act_entry(d, (uint32_t)k);
   } else {
     for (int k = t0; k < S1 * S1; k += n) {
       const uint32_t a = (uint32_t)(k % S1), b = (uint32_t)(k / S1);
-      uint32_t x = 0;
-      for (uint32_t c = 0; c < 3u; ++c) x |= patch_delta(d, a, b, c) << (8u * c);
-      T.rule[16u * b + a] =
-          make_uint2(x, reinterpret_cast<const uint32_t*>(d.trans)[kTransPairs + a * (uint32_t)S1 + b]);
+      T.rule[16u * b + a] = patch_rule_entry(d, a, b);
     }
   }
 }
@@ -168,7 +178,8 @@ __device__ __forceinline__ uint32_t patch_mirror(uint32_t e, int w, int h, int l
 // pair).  PL = 1: A the action's fields; PL = 2: A.x = 8 * action, A.y the
 // action draw.  Almost every attempt of a large lattice with movement is an
 // exchange (epsilon = 2 M N), so four exchanges take a path of their own:
-// four logic operations a step instead of ten.
+// four logic operations a step instead of ten.  (A choice per step was
+// slower: its branches cost more than the steps they shorten.)
 template <int PL>
 struct Steps2 {
   uint2 L[4], A[4];
@@ -383,7 +394,8 @@ struct StepKeys {
   uint32_t z3, w3;
 };
 
-__host__ __device__ __forceinline__ StepKeys step_keys(uint32_t m, const uint32_t* __restrict__ rk) {
+template <class RK>
+__host__ __device__ __forceinline__ StepKeys step_keys(uint32_t m, RK rk) {
   const uint64_t p1 = (uint64_t)0xCD9E8D57u * m;
   const uint64_t q1 = (uint64_t)0xCD9E8D57u * (kTagStep ^ rk[1]);          // round 2, third word of round 1
   const uint32_t x2 = (uint32_t)(q1 >> 32) ^ (uint32_t)p1 ^ rk[2];         // round 2, first word
@@ -397,7 +409,8 @@ __host__ __device__ __forceinline__ StepKeys step_keys(uint32_t m, const uint32_
 }
 
 // philox10_rk((0, g, m, STEP)) from the keys of MCS m.
-__host__ __device__ __forceinline__ uint4 philox_step(const StepKeys& k, uint32_t g, const uint32_t* __restrict__ rk) {
+template <class RK>
+__host__ __device__ __forceinline__ uint4 philox_step(const StepKeys& k, uint32_t g, RK rk) {
   const uint64_t p0 = (uint64_t)0xD2511F53u * (k.x1 ^ g);                  // round 2
   const uint64_t p1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(p0 >> 32) ^ rk[3]);   // round 3
   uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ k.x3, (uint32_t)p1, k.z3 ^ (uint32_t)p0, k.w3);
@@ -409,6 +422,62 @@ __host__ __device__ __forceinline__ uint4 philox_step(const StepKeys& k, uint32_
                    (uint32_t)a);
   }
   return c;
+}
+
+// One sub-block of a fine phase with what is known of it before the phase:
+// for a 2 x 2 one its steps, for one with a 3-site side its random words, in
+// the same registers (word t in s.L[t / 2], the last one in i8).
+template <int PL>
+struct PatchItem {
+  Steps2<PL> s;
+  uint32_t i8;
+  int i00, dc, dr;
+  uint32_t fl;   // 1 present, 2 three wide, 4 three high, edge flags << 4
+};
+
+// The random words of sub-block g in MCS m and, for a 2 x 2 one, its steps;
+// fl and the macro indexes are set.
+template <int PL, int LG, bool REFLECT, class RK>
+__device__ __forceinline__ void patch_item_draw(PatchItem<PL>& I, const StepKeys& key, uint32_t g, uint32_t m,
+                                                RK rk, const PatchTables& T, uint32_t tx, uint32_t txi) {
+  if (!(I.fl & 6u)) {
+    I.s = patch_steps2<PL, LG, REFLECT>(philox_step(key, g, rk), T, tx, txi, REFLECT ? I.fl >> 4 : 0u);
+  } else {
+    // the three calls side by side, also where a 2 x 3 sub-block needs two:
+    // the phase waits for the 3 x 3 one
+    uint4 x = make_uint4(0u, g, m, kTagStep), y = x, z = x;
+    y.x = 1u;
+    z.x = 2u;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+      x = philox_round(x, rk[2 * r], rk[2 * r + 1]);
+      y = philox_round(y, rk[2 * r], rk[2 * r + 1]);
+      z = philox_round(z, rk[2 * r], rk[2 * r + 1]);
+    }
+    I.s.L[0] = make_uint2(x.x, x.y);
+    I.s.L[1] = make_uint2(x.z, x.w);
+    I.s.L[2] = make_uint2(y.x, y.y);
+    I.s.L[3] = make_uint2(y.z, y.w);
+    I.i8 = z.x;
+  }
+}
+
+// All its attempts, from and to its macros.
+template <int PL, int LG, bool REFLECT>
+__device__ __forceinline__ void patch_item_run(typename MacroOf<PL>::type* __restrict__ M, int pitch,
+                                               const PatchItem<PL>& I, const PatchTables& T, uint32_t tx,
+                                               uint32_t txi) {
+  if (!(I.fl & 6u)) {
+    uint32_t v[PL];
+    patch_load2<PL>(M, I.i00, I.dc, I.dr, v);
+    patch_run2<PL>(v, I.s, T);
+    patch_store2<PL>(M, I.i00, I.dc, I.dr, v);
+  } else {
+    const uint32_t w[9] = {I.s.L[0].x, I.s.L[0].y, I.s.L[1].x, I.s.L[1].y, I.s.L[2].x, I.s.L[2].y, I.s.L[3].x,
+                           I.s.L[3].y, I.i8};
+    patch_irregular<PL, LG, REFLECT>(M, I.i00, I.dc, I.dr, pitch, (I.fl & 2u) != 0u, (I.fl & 4u) != 0u, w, T, tx, txi,
+                                     REFLECT ? I.fl >> 4 : 0u);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -474,5 +543,11 @@ __host__ __device__ inline void axis_quad(const AxisGeom& g, int P, int k2, int&
   const int irr = a ? ia : ib;
   pos = q >= irr ? na * (ha - ia) + (i - na) * (hb - ib) + (q - irr) : regular + na * ia + (i - na) * ib + q;
 }
+
+// Reciprocal of quot_rcp (0: d = 1, no division).
+__host__ __device__ inline uint32_t quot_rcp_of(int d) { return d <= 1 ? 0u : 0xFFFFFFFFu / (uint32_t)d + 1u; }
+// floor(n / d) for n d < 2^32 from ceil(2^32 / d) (0 for d = 1): the product
+// overshoots n / d by less than n / 2^32 < 1 / d.
+__device__ __forceinline__ uint32_t quot_rcp(uint32_t n, uint32_t rcp) { return rcp ? __umulhi(n, rcp) : n; }
 
 }  // namespace escg_impl

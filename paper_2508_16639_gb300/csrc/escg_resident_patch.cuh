@@ -60,7 +60,7 @@ __host__ __device__ inline ResidentLayout resident_layout(const LatticeDesc& d, 
 }
 
 // Sub-blocks of one fine phase, at most (the threads a launch can use).
-inline int resident_phase_items(const LatticeDesc& d) {
+__host__ __device__ inline int resident_phase_items(const LatticeDesc& d) {
   int n = 0;
   for (int cy = 0; cy < 2; ++cy)
     for (int cx = 0; cx < 2; ++cx) {
@@ -124,24 +124,19 @@ __device__ __forceinline__ void resident_setup(const LatticeDesc& d, const Resid
                 reinterpret_cast<uint32_t*>(dyn + R.slx), reinterpret_cast<uint16_t*>(dyn + R.mapx), S.nq[0], S.nr[0]);
   resident_axis(d.ay, d.Py, d.H, d.reflect != 0, reinterpret_cast<uint32_t*>(dyn + R.segy), reinterpret_cast<uint32_t*>(dyn + R.quady),
                 reinterpret_cast<uint32_t*>(dyn + R.sly), reinterpret_cast<uint16_t*>(dyn + R.mapy), S.nq[1], S.nr[1]);
-  auto rcp = [](int n) { return n <= 1 ? 0u : 0xFFFFFFFFu / (uint32_t)n + 1u; };   // 0: n = 1, no division
   if (threadIdx.x < 2) {
     int t, r;
     axis_quads(d.ax, d.P, (int)threadIdx.x, &t, &r);
-    S.rcp_nq[threadIdx.x] = rcp(t);
-    S.rcp_ni[threadIdx.x] = rcp(t - r);
+    S.rcp_nq[threadIdx.x] = quot_rcp_of(t);
+    S.rcp_ni[threadIdx.x] = quot_rcp_of(t - r);
   }
   if (threadIdx.x < 4) {
     int tx, rx, ty, ry;
     axis_quads(d.ax, d.P, (int)(threadIdx.x & 1u), &tx, &rx);
     axis_quads(d.ay, d.Py, (int)(threadIdx.x >> 1), &ty, &ry);
-    S.col[threadIdx.x] = make_uint4((uint32_t)(tx * ty), (uint32_t)(rx * ry), (uint32_t)rx, rcp(rx));
+    S.col[threadIdx.x] = make_uint4((uint32_t)(tx * ty), (uint32_t)(rx * ry), (uint32_t)rx, quot_rcp_of(rx));
   }
 }
-
-// floor(n / d) for n d < 2^32 from ceil(2^32 / d) (0 for d = 1): the product
-// overshoots n / d by less than n / 2^32 < 1 / d.
-__device__ __forceinline__ uint32_t quot_rcp(uint32_t n, uint32_t rcp) { return rcp ? __umulhi(n, rcp) : n; }
 
 __device__ __forceinline__ uint32_t load_site(const LatticeDesc& d, uint32_t row, uint32_t col) {
   const uint8_t* p = d.lat + (size_t)row * d.pitch;
@@ -201,19 +196,23 @@ __device__ __forceinline__ void resident_drain(const LatticeDesc& d, const Resid
   }
 }
 
+// Barrier of the nthr threads that run a resident lattice (barriers 1 .. 8 hand
+// its phases on).
+__device__ __forceinline__ void res_sync(uint32_t nthr) { bar_named(14u, nthr); }
+
 // Species histogram of the macros into S.hist.  Unused fields hold 0, so the
 // empty sites are counted as the rest.
 template <int PL>
 __device__ __forceinline__ void resident_count_macros(const LatticeDesc& d, const ResidentLayout& R, const uint8_t* dyn,
-                                                      ResidentPatchSmem& S) {
+                                                      ResidentPatchSmem& S, uint32_t nthr) {
   if (threadIdx.x < kMaxStates) S.hist[threadIdx.x] = 0;
-  __syncthreads();
+  res_sync(nthr);
   const uint32_t* W = reinterpret_cast<const uint32_t*>(dyn);
   const int words = R.nsy * R.pitch * PL / 4;
   uint32_t c[kMaxStates];
 #pragma unroll
   for (int v = 0; v < kMaxStates; ++v) c[v] = 0;
-  for (int k = threadIdx.x; k < words; k += blockDim.x) {
+  for (int k = threadIdx.x; k < words; k += (int)nthr) {
     const uint32_t x = W[k];
 #pragma unroll
     for (int v = 1; v < (PL == 1 ? 4 : kMaxStates); ++v) {
@@ -234,29 +233,19 @@ __device__ __forceinline__ void resident_count_macros(const LatticeDesc& d, cons
     const uint32_t s = __reduce_add_sync(0xFFFFFFFFu, c[v]);
     if (lane == 0 && s) atomicAdd(&S.hist[v], s);
   }
-  __syncthreads();
+  res_sync(nthr);
   if (threadIdx.x == 0) {
     uint32_t rest = (uint32_t)(d.L * d.H);
     for (int v = 1; v <= d.S; ++v) rest -= S.hist[v];
     S.hist[0] = rest;
   }
-  __syncthreads();
+  res_sync(nthr);
 }
-
-// One sub-block of a fine phase with what is known of it before the phase.
-template <int PL>
-struct ResidentItem {
-  Steps2<PL> s;   // 2 x 2
-  uint4 x0, x1;   // a 3-site side: the words
-  uint32_t x2;
-  int i00, dc, dr;
-  uint32_t fl;   // 1 present, 2 three wide, 4 three high, edge flags << 4
-};
 
 // Threads of a group (whole warps) and of a launch of at most max_threads: a
 // power of two of groups, so that a group takes the same phases of every MCS.
 constexpr int kResMaxGroups = 8;
-inline void resident_threads(const LatticeDesc& d, int max_threads, int* gs, int* nt) {
+__host__ __device__ inline void resident_threads(const LatticeDesc& d, int max_threads, int* gs, int* nt) {
   int g = (resident_phase_items(d) + 31) & ~31;
   if (g > max_threads) g = max_threads;
   int k = 1;
@@ -265,12 +254,13 @@ inline void resident_threads(const LatticeDesc& d, int max_threads, int* gs, int
   *nt = k * g;
 }
 
-// MCS [m_begin, m_end) on the resident macros, by blockDim.x / gs groups of gs
-// threads; on_log as in resident_run of the one-byte image.  Returns the MCS
+// MCS [m_begin, m_end) on the resident macros, by threads 0 .. nthr - 1 in groups of
+// gs; rk: the round keys; on_log as in resident_run of the
+// one-byte image.  Returns the MCS
 // reached.
-template <int PL, int LG, bool REFLECT, class OnLog>
-__device__ uint32_t resident_run_patch(const LatticeDesc& d, const ResidentLayout& R, uint8_t* dyn,
-                                       ResidentPatchSmem& S, int gs, uint32_t m_begin, uint32_t m_end,
+template <int PL, int LG, bool REFLECT, class RK, class OnLog>
+__device__ uint32_t resident_run_patch(const LatticeDesc& d, RK rk, const ResidentLayout& R, uint8_t* dyn,
+                                       ResidentPatchSmem& S, int gs, uint32_t nthr, uint32_t m_begin, uint32_t m_end,
                                        uint32_t log_every, OnLog on_log) {
   typedef typename MacroOf<PL>::type MT;
   MT* M = reinterpret_cast<MT*>(dyn);
@@ -279,14 +269,14 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, const ResidentLayou
   const uint32_t* quadx = reinterpret_cast<const uint32_t*>(dyn + R.quadx);
   const uint32_t* quady = reinterpret_cast<const uint32_t*>(dyn + R.quady);
   uint8_t* fo = dyn + R.fo;
-  const int grp = (int)threadIdx.x / gs, tid = (int)threadIdx.x - grp * gs, groups = (int)blockDim.x / gs;
+  const int grp = (int)threadIdx.x / gs, tid = (int)threadIdx.x - grp * gs, groups = (int)nthr / gs;
   const int nblk = d.P * d.Py, pitch = R.pitch;
   const uint32_t tx = d.tx, txi = d.txi, GQ = (uint32_t)d.GQ;
   const uint32_t GQy = (uint32_t)(d.ay.r * d.ay.Qa + (d.Py - d.ay.r) * d.ay.Qb);
 
   // item `it` of fine phase fi of coarse colour `colour` in MCS m
   auto prepare = [&](int it, int colour, int fi, uint32_t m, const StepKeys& key) {
-    ResidentItem<PL> I;
+    PatchItem<PL> I;
     const int cx = colour & 1, cy = colour >> 1;
     const uint4 cp = S.col[colour];
     I.fl = it < (int)cp.x ? 1u : 0u;
@@ -327,55 +317,35 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, const ResidentLayou
         I.fl |= (ky == 0u ? 16u : 0u) | (ky == GQy - 1u ? 32u : 0u) | (kx == 0u ? 64u : 0u) | (kx == GQ - 1u ? 128u : 0u);
     }
     const uint32_t g = ky * GQ + kx;
-    const uint4 x = philox_step(key, g, d.rk);
-    if (!(I.fl & 6u)) {
-      I.s = patch_steps2<PL, LG, REFLECT>(x, S.T, tx, txi, REFLECT ? I.fl >> 4 : 0u);
-    } else {
-      I.x0 = x;
-      I.x1 = philox10_rk(make_uint4(1u, g, m, kTagStep), d.rk);
-      I.x2 = (I.fl & 6u) == 6u ? philox10_rk(make_uint4(2u, g, m, kTagStep), d.rk).x : 0u;
-    }
+    patch_item_draw<PL, LG, REFLECT>(I, key, g, m, rk, S.T, tx, txi);
     return I;
-  };
-
-  auto execute = [&](const ResidentItem<PL>& I) {
-    if (!(I.fl & 6u)) {
-      uint32_t v[PL];
-      patch_load2<PL>(M, I.i00, I.dc, I.dr, v);
-      patch_run2<PL>(v, I.s, S.T);
-      patch_store2<PL>(M, I.i00, I.dc, I.dr, v);
-    } else {
-      const uint32_t w[9] = {I.x0.x, I.x0.y, I.x0.z, I.x0.w, I.x1.x, I.x1.y, I.x1.z, I.x1.w, I.x2};
-      patch_irregular<PL, LG, REFLECT>(M, I.i00, I.dc, I.dr, pitch, (I.fl & 2u) != 0u, (I.fl & 4u) != 0u, w, S.T, tx,
-                                       txi, REFLECT ? I.fl >> 4 : 0u);
-    }
   };
 
   auto orders = [&](uint32_t m, int t, int n) {   // the blocks' fine orders of MCS m
     for (int b = t; b < nblk; b += n)
       fo[(m & 1u) * nblk + b] =
-          (uint8_t)colour_order(philox10_rk(make_uint4(0u, (uint32_t)b, m, kTagFineOrder), d.rk).x, d.perm24);
+          (uint8_t)colour_order(philox10_rk(make_uint4(0u, (uint32_t)b, m, kTagFineOrder), rk).x, d.perm24);
   };
   auto order = [&](uint32_t m) {
-    return colour_order(philox10_rk(make_uint4(0u, 0u, m, kTagOrder), d.rk).x, d.perm24);
+    return colour_order(philox10_rk(make_uint4(0u, 0u, m, kTagOrder), rk).x, d.perm24);
   };
 
-  orders(m_begin, (int)threadIdx.x, (int)blockDim.x);
+  orders(m_begin, (int)threadIdx.x, (int)nthr);
   uint32_t ord = order(m_begin);
-  StepKeys key = step_keys(m_begin, d.rk);
-  __syncthreads();
-  ResidentItem<PL> cur = prepare(tid, order_at(ord, grp >> 2), grp & 3, m_begin, key);
+  StepKeys key = step_keys(m_begin, rk);
+  res_sync(nthr);
+  PatchItem<PL> cur = prepare(tid, order_at(ord, grp >> 2), grp & 3, m_begin, key);
   bool handed = false;   // the last phase ended with a CTA barrier instead of a hand-over
   uint32_t m = m_begin;
   for (; m < m_end; ++m) {
     const uint32_t ord_next = order(m + 1u);
-    const StepKeys key_next = step_keys(m + 1u, d.rk);
+    const StepKeys key_next = step_keys(m + 1u, rk);
     const bool log_point = ((m + 1u) % log_every) == 0u, joined = log_point || m + 1u == m_end;
 #pragma unroll 1
     for (int ph = grp; ph < 16; ph += groups) {
       // the macros as the phase before left them
       if (groups == 1)
-        __syncthreads();
+        res_sync(nthr);
       else if (ph > 0 || handed)
         bar_named((uint32_t)(1 + grp), (uint32_t)(2 * gs));
       const int colour = order_at(ord, ph >> 2), fi = ph & 3;
@@ -386,7 +356,7 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, const ResidentLayou
       for (int it = tid;; it += gs) {
         // the macros first, then what the other groups' phases hide
         const bool more = it + gs < n;
-        if (cur.fl) execute(cur);
+        if (cur.fl) patch_item_run<PL, LG, REFLECT>(M, pitch, cur, S.T, tx, txi);
         if (groups > 1 && !more && !(joined && ph == 15))
           bar_arrive((uint32_t)(1 + (grp + 1) % groups), (uint32_t)(2 * gs));
         const bool nm = wrap && !more;
@@ -402,17 +372,17 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, const ResidentLayou
     ord = ord_next;
     key = key_next;
     if (log_point) {
-      __syncthreads();
-      resident_count_macros<PL>(d, R, dyn, S);
+      res_sync(nthr);
+      resident_count_macros<PL>(d, R, dyn, S, nthr);
       if (threadIdx.x == 0) S.stop = on_log(m + 1u, S.hist) ? 1u : 0u;
-      __syncthreads();
+      res_sync(nthr);
       if (S.stop) {
         ++m;
         break;
       }
     }
   }
-  __syncthreads();
+  res_sync(nthr);
   return m;
 }
 

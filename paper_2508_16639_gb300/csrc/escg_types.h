@@ -108,9 +108,9 @@ struct LatticeDesc {
   int32_t bits;         // bits per site in `lat`: 8 (one byte) or 4, 2 (packed
                         // rows: site c at bits [c*bits, (c+1)*bits), little endian)
   uint8_t perm24[24];   // the 24 colour orders, lexicographic (4 x 2 bits)
-  int32_t blocks64;     // all blocks 64x64 and all sub-blocks 2x2, whatever the rule
+  int16_t blocks64;     // all blocks 64x64 and all sub-blocks 2x2, whatever the rule
                         // and the storage (uniform64: the von Neumann, periodic rule)
-  int32_t certain;      // every dominance edge certain (no pair's interaction
+  int16_t certain;      // every dominance edge certain (no pair's interaction
                         // threshold below txi): with S <= 3 a step's rule fits
                         // a 64-bit word (escg_patch.cuh)
 };
