@@ -36,6 +36,7 @@
 #include "escg_device.cuh"
 #include "escg_internal.h"
 #include "escg_resident.cuh"
+#include "escg_resident_patch.cuh"
 #include "escg_rule8.cuh"
 #include "escg_tma.cuh"
 
@@ -47,7 +48,7 @@ struct SlotDesc {
   uint32_t max_mcs;     // budget: absolute MCS number to stop at
   int32_t stop_at_extinction;
   int32_t nb4;          // blocks per coarse phase = P*P/4 in the chunk kernel's table (0: resident)
-  int32_t rclass;       // 0: chunk kernel; 1..3: whole-lattice residency class
+  int32_t rclass;       // 0: chunk kernel; 1..3: whole-lattice residency class; kPatchClass: residency on macros
 };
 
 struct SlotState {
@@ -63,9 +64,16 @@ struct BatchCtl {
   uint32_t n_active, tot4, chunk, ticket;
   uint32_t exited, error, abort, n_admit;
   uint32_t last_chunk;  // MCS the previous batch_kernel launch covered
-  uint32_t res_ticket[3];  // dispensers of the resident kernels (classes 1..3)
-  uint32_t pad[4];
+  uint32_t res_ticket[4];  // dispensers of the resident kernels (classes 1..4)
+  uint32_t pad[3];
 };
+
+// Class of the replicas of 2 x 2 coarse blocks (L < 192), which either kernel
+// runs.  One block of a colour is all that can run at a time in them, so a
+// CTA that keeps the lattice loses no parallelism to the chunk kernel and
+// pays none of the round trips of its visits; but it issues more
+// instructions, so it pays only while SMs are idle (engine_plan).
+constexpr int kPatchClass = 4;
 
 struct BatchArgs {
   const SlotDesc* slots;
@@ -123,7 +131,8 @@ constexpr int kCompactThreads = 1024;
 __global__ void __launch_bounds__(kCompactThreads) batch_compact_kernel(const SlotDesc* slots, SlotState* states,
                                                                         BatchCtl* ctl, uint32_t* active,
                                                                         uint32_t* active_tmp, uint32_t* table,
-                                                                        const uint32_t* admit, uint32_t chunk) {
+                                                                        const uint32_t* admit, uint32_t chunk,
+                                                                        int patch_on) {
   __shared__ uint32_t s_scan[kCompactThreads];
   __shared__ uint32_t s_keep_total, s_n_old, s_n_admit, s_last;
   const int t = threadIdx.x;
@@ -171,7 +180,10 @@ __global__ void __launch_bounds__(kCompactThreads) batch_compact_kernel(const Sl
   const uint32_t per2 = (n_new + kCompactThreads - 1) / kCompactThreads;
   const uint32_t lo2 = t * per2, hi2 = min(n_new, lo2 + per2);
   uint32_t sum = 0;
-  for (uint32_t a = lo2; a < hi2; ++a) sum += (uint32_t)slots[active_tmp[a]].nb4;
+  auto entries = [&](uint32_t s) {
+    return patch_on && slots[s].rclass == kPatchClass ? 0u : (uint32_t)slots[s].nb4;
+  };
+  for (uint32_t a = lo2; a < hi2; ++a) sum += entries(active_tmp[a]);
   __syncthreads();
   s_scan[t] = sum;
   __syncthreads();
@@ -185,7 +197,7 @@ __global__ void __launch_bounds__(kCompactThreads) batch_compact_kernel(const Sl
   for (uint32_t a = lo2; a < hi2; ++a) {
     const uint32_t s = active_tmp[a];
     active[a] = s;
-    const uint32_t nb4 = (uint32_t)slots[s].nb4;
+    const uint32_t nb4 = entries(s);
     for (uint32_t j = 0; j < nb4; ++j) table[e++] = (s << 16) | j;
   }
   __syncthreads();
@@ -196,7 +208,7 @@ __global__ void __launch_bounds__(kCompactThreads) batch_compact_kernel(const Sl
     ctl->ticket = 0;
     ctl->exited = 0;
     ctl->n_admit = 0;
-    ctl->res_ticket[0] = ctl->res_ticket[1] = ctl->res_ticket[2] = 0;
+    for (int c = 0; c < 4; ++c) ctl->res_ticket[c] = 0;
     ctl->last_chunk = 0;   // consumed; the next batch_kernel launch sets it
   }
 }
@@ -386,6 +398,87 @@ __global__ void __launch_bounds__(THREADS, 65536 / (THREADS * 64)) batch_residen
       return stop;
     });
     resident_store(d, img, sp);
+    __syncthreads();
+  }
+}
+
+// Residency on macros (escg_resident_patch.cuh): a CTA takes the active
+// replicas of kPatchClass from the dispenser and runs each one's chunk.  Bound
+// by the chain of fine phases, so the CTA is as large as the SMs allow (groups
+// of threads take the phases in turn).
+template <int PL>
+__device__ __forceinline__ void batch_patch_chunk(const SlotDesc& sd, SlotState* st, uint8_t* dyn, ResidentPatchSmem& S,
+                                                  ResidentLayout& R, uint32_t m0, uint32_t m_end, uint32_t log_every) {
+  const LatticeDesc& d = sd.d;
+  if (threadIdx.x == 0) R = resident_layout(d, PL);
+  __syncthreads();
+  resident_setup<PL>(d, R, dyn, S);
+  __syncthreads();
+  resident_fill<PL>(d, R, dyn);
+  __syncthreads();
+  int gs, nthr;
+  resident_threads(d, (int)blockDim.x, &gs, &nthr);
+  if ((int)threadIdx.x < nthr)
+    resident_run_patch<PL, 2, false>(d, AddKeys{d.key0, d.key1}, R, dyn, S, gs, (uint32_t)nthr, m0, m_end, log_every,
+                                     [&](uint32_t mm, const uint32_t* hist) {
+      int alive = 0;
+      for (int v = 0; v < kMaxStates; ++v) {
+        const unsigned long long c = (v <= d.S) ? hist[v] : 0ull;
+        st->counts[v] = c;
+        if (v >= 1 && v <= d.S && c > 0) ++alive;
+      }
+      st->counts_mcs = mm;
+      const bool stop = sd.stop_at_extinction && alive <= 1;
+      if (stop) st->stopped = 1;
+      return stop;
+    });
+  __syncthreads();
+  resident_drain<PL>(d, R, dyn);
+}
+
+template <int THREADS>   // 1024 or 512
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) batch_patch_kernel(BatchArgs a, const uint32_t* active) {
+  extern __shared__ __align__(16) uint8_t res_dyn[];
+  __shared__ ResidentPatchSmem S;
+  __shared__ ResidentLayout R;
+  __shared__ SlotDesc sd;
+  __shared__ uint32_t s_slot, s_quit;
+  BatchCtl* ctl = a.ctl;
+  const int tid = threadIdx.x;
+  const uint32_t n_active = ctl->n_active, chunk = ctl->chunk;
+  for (;;) {
+    if (tid == 0) {
+      uint32_t quit = 0, s = 0;
+      for (;;) {
+        const uint32_t t = atomicAdd(&ctl->res_ticket[kPatchClass - 1], 1u);
+        if (t >= n_active || b_ld_volatile(&ctl->abort)) {
+          quit = 1;
+          break;
+        }
+        s = active[t];
+        if (a.slots[s].rclass == kPatchClass) break;
+      }
+      s_slot = s;
+      s_quit = quit;
+    }
+    __syncthreads();
+    if (s_quit) break;
+    {
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(a.slots + s_slot);
+      uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
+      for (int w = tid; w < (int)(sizeof(SlotDesc) / 4); w += THREADS) dst[w] = src[w];
+    }
+    __syncthreads();
+    SlotState* st = a.states + s_slot;
+    const uint32_t m0 = st->mcs, m_end = min(m0 + chunk, sd.max_mcs);
+    if (m0 < m_end) {   // uniform: every thread read the same words
+      if (sd.d.S <= 3 && sd.d.certain)
+        batch_patch_chunk<1>(sd, st, res_dyn, S, R, m0, m_end, a.log_every);
+      else
+        batch_patch_chunk<2>(sd, st, res_dyn, S, R, m0, m_end, a.log_every);
+      // the chunk kernel may run the replica's next chunk
+      if (tid < sd.d.P * sd.d.Py) sd.done[tid] = m_end;
+    }
     __syncthreads();
   }
 }
@@ -931,8 +1024,14 @@ struct Engine {
   bool resident = false;          // whole-lattice residency for replicas that fit
   int res_bytes3 = 0;             // dynamic shared memory of class 3
   int grid_res[4] = {0, 0, 0, 0};
+  int n_patch = 0;                // slots of kPatchClass in use
+  int patch_bytes = 0;            // dynamic shared memory of batch_patch_kernel
+  int n_used = 0;                 // slots in use
+  int sms = 0;
+  bool patch_on = false;          // batch_patch_kernel runs the replicas of kPatchClass
   uint64_t launches = 0;
   cudaGraphExec_t graph = nullptr;
+  int graph_patch = 0;            // replicas batch_patch_kernel runs in it
   uint32_t spin_limit = 2000000;
   static constexpr int kGraphChunks = 16;
 };
@@ -973,10 +1072,19 @@ cudaError_t launch_resident_kernels(Engine* e) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_patch(Engine* e) {
+  BatchArgs a{e->d_slots, e->d_states, e->d_ctl, e->d_table, e->log_every, e->spin_limit};
+  if (e->n_patch <= e->sms)
+    batch_patch_kernel<1024><<<e->n_patch, 1024, e->patch_bytes, e->stream>>>(a, e->d_active);
+  else
+    batch_patch_kernel<512><<<e->n_patch, 512, e->patch_bytes, e->stream>>>(a, e->d_active);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_compact(Engine* e) {
   batch_compact_kernel<<<1, kCompactThreads, 0, e->stream>>>(e->d_slots, e->d_states, e->d_ctl, e->d_active,
                                                              e->d_active_tmp, e->d_table, e->d_admit,
-                                                             e->log_every);
+                                                             e->log_every, e->patch_on ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1052,6 +1160,13 @@ int engine_init(Engine* e, int max_slots, size_t arena_bytes, size_t table_cap, 
   e->grid_tma[1] = sms * (per < 1 ? 1 : per);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_tma_kernel<256>, 256 + 32, 0);
   e->grid_tma[2] = sms * (per < 1 ? 1 : per);
+  e->sms = sms;
+  for (int L = 8; L < 192; ++L) {   // the replicas of 2 x 2 coarse blocks
+    const AxisGeom g = make_axis_geom(L, 2);
+    if (slot_axis_ok(g)) e->patch_bytes = std::max(e->patch_bytes, resident_layout(g, 2, L, g, 2, L, 2).bytes);
+  }
+  cudaFuncSetAttribute(batch_patch_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, e->patch_bytes);
+  cudaFuncSetAttribute(batch_patch_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, e->patch_bytes);
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, e->device);
   e->res_bytes3 = optin - (int)(sizeof(ResidentSmem) + sizeof(SlotDesc)) - 256;
@@ -1137,6 +1252,8 @@ int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int s
     const int bytes = resident_dyn_bytes(sp.L, sp.L);
     sd.rclass = bytes <= kResBytes1 ? 1 : (bytes <= kResBytes2 ? 2 : (bytes <= e->res_bytes3 ? 3 : 0));
     if (sd.rclass) sd.nb4 = 0;   // not in the chunk kernel's table
+  } else if (p.P == 2 && slot_axis_ok(d.ax)) {
+    sd.rclass = kPatchClass;     // its table entries stay: see engine_plan
   }
   CUtensorMap map;
   if (!encode_lattice_map(&map, d.lat, d.L, d.pitch, kBSP, kBRows)) {
@@ -1166,6 +1283,8 @@ int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int s
     return ESCG_ECUDA;
   }
   e->launches += 2;
+  if (sd.rclass == kPatchClass) e->n_patch++;
+  e->n_used++;
   e->h_slots[slot] = sd;
   e->slot_off[slot] = off;
   e->slot_bytes[slot] = pl.bytes;
@@ -1174,7 +1293,11 @@ int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int s
 }
 
 void engine_release(Engine* e, int slot) {
-  if (e->slot_bytes[slot]) e->arena.release(e->slot_off[slot], e->slot_bytes[slot]);
+  if (e->slot_bytes[slot]) {
+    if (e->h_slots[slot].rclass == kPatchClass) e->n_patch--;
+    e->n_used--;
+    e->arena.release(e->slot_off[slot], e->slot_bytes[slot]);
+  }
   e->slot_bytes[slot] = 0;
 }
 
@@ -1203,12 +1326,12 @@ int engine_flush_admits(Engine* e) {
 // One chunk: compaction, the resident kernels, then the chunk kernel (whose
 // last CTA records how far the launch advanced the replicas).
 int engine_chunk(Engine* e, int threads) {
-  if (launch_compact(e) != cudaSuccess || launch_resident_kernels(e) != cudaSuccess ||
-      launch_batch_kernel(e, threads) != cudaSuccess) {
+  if (launch_compact(e) != cudaSuccess || (e->patch_on && launch_patch(e) != cudaSuccess) ||
+      launch_resident_kernels(e) != cudaSuccess || launch_batch_kernel(e, threads) != cudaSuccess) {
     set_last_error("chunk launch failed");
     return ESCG_ECUDA;
   }
-  e->launches += e->resident ? 5 : 2;
+  e->launches += (e->resident ? 5 : 2) + (e->patch_on ? 1 : 0);
   return ESCG_OK;
 }
 
@@ -1250,7 +1373,14 @@ int engine_autotune(Engine* e, uint64_t* chunks_left) {
 }
 
 int engine_build_graph(Engine* e) {
+  // a graph holds the launches of batch_patch_kernel as they were planned
+  const int patch = e->patch_on ? e->n_patch : 0;
+  if (e->graph && patch != e->graph_patch) {
+    cudaGraphExecDestroy(e->graph);
+    e->graph = nullptr;
+  }
   if (!e->use_graph || e->graph) return ESCG_OK;
+  e->graph_patch = patch;
   cudaGraph_t g;
   if (cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     set_last_error("CUDA graph capture failed to start");
@@ -1258,6 +1388,7 @@ int engine_build_graph(Engine* e) {
   }
   for (int c = 0; c < Engine::kGraphChunks; ++c) {
     launch_compact(e);
+    if (e->patch_on) launch_patch(e);
     launch_resident_kernels(e);
     launch_batch_kernel(e, e->threads);
   }
@@ -1280,12 +1411,21 @@ int engine_active(Engine* e, uint32_t* out) {
   return ESCG_OK;
 }
 
+// Which kernel runs the replicas of kPatchClass.  Resident while no other
+// replica is in the engine and each has half an SM to itself: us per MCS,
+// chunk kernel -> resident, 144 replicas of L = 100, S = 8 43.4 -> 22.7, 138 of
+// L = 64 and 100 42.4 -> 22.8, 8 of them 38.9 -> 22.1; with 518 of them 47.5 -> 58.9,
+// with 576 of L = 100 51.1 -> 64.7, and beside larger replicas, whose visits need
+// the issue slots, 256 of all sizes 74.7 -> 81.0.
+void engine_plan(Engine* e) { e->patch_on = e->n_patch > 0 && e->n_patch == e->n_used && e->n_patch <= 2 * e->sms; }
+
 // Runs up to `chunks` chunks (0: until no replica is active), stopping early
 // when the active set empties; ends with a compaction so that every
 // replica's MCS number and retirement are settled.
 int engine_run(Engine* e, uint64_t chunks, bool until_idle) {
   int rc = engine_flush_admits(e);
   if (rc != ESCG_OK) return rc;
+  engine_plan(e);
   uint64_t left = chunks;
   if (e->threads == 0) {
     rc = engine_autotune(e, &left);
@@ -1301,7 +1441,7 @@ int engine_run(Engine* e, uint64_t chunks, bool until_idle) {
         set_last_error("graph launch failed");
         return ESCG_ECUDA;
       }
-      e->launches += (e->resident ? 5 : 2) * G;
+      e->launches += ((e->resident ? 5 : 2) + (e->graph_patch ? 1 : 0)) * G;
       left = left >= G ? left - G : 0;
       group = true;
     } else {
