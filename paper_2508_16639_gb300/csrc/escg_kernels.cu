@@ -1612,7 +1612,8 @@ bool resident_fits(const LatticeDesc& d, int device) {
 // one-byte image; every other lattice that fits runs on macros, whose image
 // is at most half as large.
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream) {
-  if (slot_axis_ok(a.d.ax) && slot_axis_ok(a.d.ay)) {
+  if (slot_axis_ok(a.d.ax) && slot_axis_ok(a.d.ay) &&
+      resident_layout(a.d, patch_planes(a.d)).bytes <= kResPatchBytes) {
     const int bytes = resident_layout(a.d, patch_planes(a.d)).bytes;
     const void* fn = resident_patch_fn(a.d);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

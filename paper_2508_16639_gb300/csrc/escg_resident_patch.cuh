@@ -25,15 +25,30 @@ struct ResidentPatchSmem {
   uint32_t hist[kMaxStates];
   uint32_t stop;
   int32_t nq[2][2], nr[2][2];   // [axis][parity]: quads and regular quads
-  uint32_t rcp_nq[2], rcp_ni[2];   // ceil(2^32 / n) of the column counts by parity
-  uint4 col[4];   // by colour: items of a fine phase, regular ones, regular columns, their reciprocal
+  int32_t n[4];                 // by colour: items of a fine phase
 };
 
-// Dynamic shared memory: the macros, then the tables of both axes.
+// Dynamic shared memory: the macros, the items' table, the tables of both axes.
+// A lattice of more than kResPatchBytes stays on the one-byte image.
+constexpr int kResPatchBytes = 222 * 1024;
 struct ResidentLayout {
   int nsx, nsy, pitch;               // slots, macros per row (whole 32-bit words)
-  int segx, segy, quadx, quady, slx, sly, mapx, mapy, fo, bytes;   // byte offsets
+  int items;                         // entries of a colour in the items' table (whole warps)
+  int table, segx, segy, quadx, quady, slx, sly, mapx, mapy, fo, bytes;   // byte offsets
 };
+
+// Sub-blocks of one fine phase, at most (the threads a launch can use).
+__host__ __device__ inline int resident_phase_items(const AxisGeom& ax, int P, const AxisGeom& ay, int Py) {
+  int n = 0;
+  for (int cy = 0; cy < 2; ++cy)
+    for (int cx = 0; cx < 2; ++cx) {
+      int qx, rx, qy, ry;
+      axis_quads(ax, P, cx, &qx, &rx);
+      axis_quads(ay, Py, cy, &qy, &ry);
+      if (qx * qy > n) n = qx * qy;
+    }
+  return n;
+}
 
 __host__ __device__ inline ResidentLayout resident_layout(const AxisGeom& ax, int P, int L, const AxisGeom& ay, int Py,
                                                           int H, int planes) {
@@ -42,8 +57,10 @@ __host__ __device__ inline ResidentLayout resident_layout(const AxisGeom& ax, in
   R.nsy = axis_slots(ay, Py);
   R.pitch = planes == 1 ? (R.nsx + 3) & ~3 : (R.nsx + 1) & ~1;
   const int gx = ax.r * ax.Qa + (P - ax.r) * ax.Qb, gy = ay.r * ay.Qa + (Py - ay.r) * ay.Qb;
+  R.items = (resident_phase_items(ax, P, ay, Py) + 31) & ~31;
   int o = (R.nsy * R.pitch * planes + 15) & ~15;
-  R.segx = o;
+  R.table = o;
+  R.segx = o += 32 * R.items;
   R.segy = o += 4 * gx;
   R.quadx = o += 4 * gy;
   R.quady = o += 2 * gx;
@@ -53,32 +70,18 @@ __host__ __device__ inline ResidentLayout resident_layout(const AxisGeom& ax, in
   R.mapy = o += 2 * ((L + 1) & ~1);
   R.fo = o += 2 * ((H + 1) & ~1);
   R.bytes = (o + 2 * P * Py + 15) & ~15;
+  if (R.nsy * R.pitch > 65536) R.bytes = 1 << 30;   // past the items' macro indexes
   return R;
 }
 __host__ __device__ inline ResidentLayout resident_layout(const LatticeDesc& d, int planes) {
   return resident_layout(d.ax, d.P, d.L, d.ay, d.Py, d.H, planes);
 }
 
-// Sub-blocks of one fine phase, at most (the threads a launch can use).
-__host__ __device__ inline int resident_phase_items(const LatticeDesc& d) {
-  int n = 0;
-  for (int cy = 0; cy < 2; ++cy)
-    for (int cx = 0; cx < 2; ++cx) {
-      int qx, rx, qy, ry;
-      axis_quads(d.ax, d.P, cx, &qx, &rx);
-      axis_quads(d.ay, d.Py, cy, &qy, &ry);
-      if (qx * qy > n) n = qx * qy;
-    }
-  return n;
-}
-
 // Tables of one axis (n sites, P blocks): segment k -> left joint slot |
 // right joint slot << 12 | 3 wide << 24; quad position -> left joint slot |
-// first segment << 12 | block / 2 << 24 | plain << 31 (both segments 2 wide,
-// the second one's right joint not wrapped and, with a reflecting boundary,
-// no segment at an edge), the quads of parity 0, then those of parity 1; slot
-// -> its sites (half 0 | half 1 << 16, 0xFFFF none); site -> 2 slot + half.
-__device__ __forceinline__ void resident_axis(const AxisGeom& g, int P, int n, bool reflect, uint32_t* seg, uint32_t* quad,
+// first segment << 12 | block / 2 << 24, the quads of parity 0, then those of
+// parity 1; slot -> its sites (half 0 | half 1 << 16, 0xFFFF none); site -> 2 slot + half.
+__device__ __forceinline__ void resident_axis(const AxisGeom& g, int P, int n, uint32_t* seg, uint32_t* quad,
                                               uint32_t* sl, uint16_t* map, int32_t* nq, int32_t* nr) {
   const int G = g.r * g.Qa + (P - g.r) * g.Qb;
   for (int k = threadIdx.x; k < G; k += blockDim.x) {
@@ -99,13 +102,10 @@ __device__ __forceinline__ void resident_axis(const AxisGeom& g, int P, int n, b
   axis_quads(g, P, 0, &t0, &r0);
   for (int k = threadIdx.x; k < G / 2; k += blockDim.x) {
     int b, s, pos, slot, first;
-    bool w0, w1;
+    bool wide;
     axis_quad(g, P, k, b, s, pos);
-    axis_segment(g, s + 1, slot, w1, first);
-    axis_segment(g, s, slot, w0, first);
-    const bool plain = !w0 && !w1 && s + 2 < G && !(reflect && s == 0);
-    quad[((b & 1) ? t0 : 0) + pos] =
-        (uint32_t)slot | ((uint32_t)s << 12) | ((uint32_t)(b >> 1) << 24) | (plain ? 1u << 31 : 0u);
+    axis_segment(g, s, slot, wide, first);
+    quad[((b & 1) ? t0 : 0) + pos] = (uint32_t)slot | ((uint32_t)s << 12) | ((uint32_t)(b >> 1) << 24);
   }
   if (threadIdx.x < 2) {
     int t, r;
@@ -120,21 +120,51 @@ template <int PL>
 __device__ __forceinline__ void resident_setup(const LatticeDesc& d, const ResidentLayout& R, uint8_t* dyn,
                                                ResidentPatchSmem& S) {
   patch_tables_fill<PL>(S.T, d, threadIdx.x, blockDim.x);
-  resident_axis(d.ax, d.P, d.L, d.reflect != 0, reinterpret_cast<uint32_t*>(dyn + R.segx), reinterpret_cast<uint32_t*>(dyn + R.quadx),
+  resident_axis(d.ax, d.P, d.L, reinterpret_cast<uint32_t*>(dyn + R.segx), reinterpret_cast<uint32_t*>(dyn + R.quadx),
                 reinterpret_cast<uint32_t*>(dyn + R.slx), reinterpret_cast<uint16_t*>(dyn + R.mapx), S.nq[0], S.nr[0]);
-  resident_axis(d.ay, d.Py, d.H, d.reflect != 0, reinterpret_cast<uint32_t*>(dyn + R.segy), reinterpret_cast<uint32_t*>(dyn + R.quady),
+  resident_axis(d.ay, d.Py, d.H, reinterpret_cast<uint32_t*>(dyn + R.segy), reinterpret_cast<uint32_t*>(dyn + R.quady),
                 reinterpret_cast<uint32_t*>(dyn + R.sly), reinterpret_cast<uint16_t*>(dyn + R.mapy), S.nq[1], S.nr[1]);
-  if (threadIdx.x < 2) {
-    int t, r;
-    axis_quads(d.ax, d.P, (int)threadIdx.x, &t, &r);
-    S.rcp_nq[threadIdx.x] = quot_rcp_of(t);
-    S.rcp_ni[threadIdx.x] = quot_rcp_of(t - r);
-  }
-  if (threadIdx.x < 4) {
-    int tx, rx, ty, ry;
-    axis_quads(d.ax, d.P, (int)(threadIdx.x & 1u), &tx, &rx);
-    axis_quads(d.ay, d.Py, (int)(threadIdx.x >> 1), &ty, &ry);
-    S.col[threadIdx.x] = make_uint4((uint32_t)(tx * ty), (uint32_t)(rx * ry), (uint32_t)rx, quot_rcp_of(rx));
+  __syncthreads();
+  // The items of each colour, a quad each: regular quads first, then the rows
+  // and the columns of the others.  x: top left macro (16 bits) | 3-site
+  // segments (columns 2 qx, 2 qx + 1 at bits 16, 17, rows at 18, 19) | last column
+  // (20) and row (21), first column (22) and row (23) of the lattice | present
+  // (31); y: sub-block of fine colour 0 | block << 24.  Worked out here once: an
+  // item is 25 instructions of a fine phase otherwise.
+  uint2* table = reinterpret_cast<uint2*>(dyn + R.table);
+  const uint32_t* segx = reinterpret_cast<const uint32_t*>(dyn + R.segx);
+  const uint32_t* segy = reinterpret_cast<const uint32_t*>(dyn + R.segy);
+  const uint32_t* quadx = reinterpret_cast<const uint32_t*>(dyn + R.quadx);
+  const uint32_t* quady = reinterpret_cast<const uint32_t*>(dyn + R.quady);
+  const int GQ = d.GQ, GQy = d.ay.r * d.ay.Qa + (d.Py - d.ay.r) * d.ay.Qb;
+  if (threadIdx.x < 4) S.n[threadIdx.x] = S.nq[0][threadIdx.x & 1u] * S.nq[1][threadIdx.x >> 1];
+  for (int i = threadIdx.x; i < 4 * R.items; i += blockDim.x) {
+    const int c = i / R.items, it = i - c * R.items, cx = c & 1, cy = c >> 1;
+    const int nqx = S.nq[0][cx], nqy = S.nq[1][cy], rx = S.nr[0][cx], ry = S.nr[1][cy];
+    uint2 v = make_uint2(0u, 0u);
+    if (it < nqx * nqy) {
+      const int k = it - rx * ry, top = nqx * (nqy - ry);
+      int px, py;
+      if (k < 0) {
+        py = it / rx;
+        px = it - py * rx;
+      } else if (k < top) {
+        py = k / nqx;
+        px = k - py * nqx;
+        py += ry;
+      } else {
+        py = (k - top) / (nqx - rx);
+        px = k - top - py * (nqx - rx) + rx;
+      }
+      const uint32_t qx = quadx[(cx ? S.nq[0][0] : 0) + px], qy = quady[(cy ? S.nq[1][0] : 0) + py];
+      const uint32_t kx = (qx >> 12) & 0xFFFu, ky = (qy >> 12) & 0xFFFu;
+      const uint32_t blk = (2u * (qy >> 24) + (uint32_t)cy) * (uint32_t)d.P + 2u * (qx >> 24) + (uint32_t)cx;
+      v.x = ((qy & 0xFFFu) * (uint32_t)R.pitch + (qx & 0xFFFu)) | (segx[kx] >> 24) << 16 | (segx[kx + 1] >> 24) << 17 |
+            (segy[ky] >> 24) << 18 | (segy[ky + 1] >> 24) << 19 | ((int)kx + 2 == GQ ? 1u << 20 : 0u) |
+            ((int)ky + 2 == GQy ? 1u << 21 : 0u) | (kx == 0u ? 1u << 22 : 0u) | (ky == 0u ? 1u << 23 : 0u) | 1u << 31;
+      v.y = (ky * (uint32_t)GQ + kx) | blk << 24;
+    }
+    table[i] = v;
   }
 }
 
@@ -246,7 +276,7 @@ __device__ __forceinline__ void resident_count_macros(const LatticeDesc& d, cons
 // power of two of groups, so that a group takes the same phases of every MCS.
 constexpr int kResMaxGroups = 8;
 __host__ __device__ inline void resident_threads(const LatticeDesc& d, int max_threads, int* gs, int* nt) {
-  int g = (resident_phase_items(d) + 31) & ~31;
+  int g = (resident_phase_items(d.ax, d.P, d.ay, d.Py) + 31) & ~31;
   if (g > max_threads) g = max_threads;
   int k = 1;
   while (2 * k <= kResMaxGroups && 2 * k * g <= max_threads) k *= 2;
@@ -264,61 +294,28 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, RK rk, const Reside
                                        uint32_t log_every, OnLog on_log) {
   typedef typename MacroOf<PL>::type MT;
   MT* M = reinterpret_cast<MT*>(dyn);
-  const uint32_t* segx = reinterpret_cast<const uint32_t*>(dyn + R.segx);
-  const uint32_t* segy = reinterpret_cast<const uint32_t*>(dyn + R.segy);
-  const uint32_t* quadx = reinterpret_cast<const uint32_t*>(dyn + R.quadx);
-  const uint32_t* quady = reinterpret_cast<const uint32_t*>(dyn + R.quady);
+  const uint2* table = reinterpret_cast<const uint2*>(dyn + R.table);
   uint8_t* fo = dyn + R.fo;
   const int grp = (int)threadIdx.x / gs, tid = (int)threadIdx.x - grp * gs, groups = (int)nthr / gs;
   const int nblk = d.P * d.Py, pitch = R.pitch;
   const uint32_t tx = d.tx, txi = d.txi, GQ = (uint32_t)d.GQ;
-  const uint32_t GQy = (uint32_t)(d.ay.r * d.ay.Qa + (d.Py - d.ay.r) * d.ay.Qb);
 
   // item `it` of fine phase fi of coarse colour `colour` in MCS m
-  auto prepare = [&](int it, int colour, int fi, uint32_t m, const StepKeys& key) {
-    PatchItem<PL> I;
-    const int cx = colour & 1, cy = colour >> 1;
-    const uint4 cp = S.col[colour];
-    I.fl = it < (int)cp.x ? 1u : 0u;
-    if (!I.fl) return I;
-    // regular quads first, then the rows and the columns of the others
-    uint32_t px, py;
-    if (it < (int)cp.y) {
-      py = quot_rcp((uint32_t)it, cp.w);
-      px = (uint32_t)it - py * cp.z;
-    } else {
-      const int nqx = S.nq[0][cx], nry = S.nr[1][cy], top = nqx * (S.nq[1][cy] - nry), k = it - (int)cp.y;
-      if (k < top) {
-        py = quot_rcp((uint32_t)k, S.rcp_nq[cx]);
-        px = (uint32_t)k - py * (uint32_t)nqx;
-        py += (uint32_t)nry;
-      } else {
-        py = quot_rcp((uint32_t)(k - top), S.rcp_ni[cx]);
-        px = (uint32_t)(k - top) - py * (uint32_t)(nqx - (int)cp.z) + cp.z;
-      }
-    }
-    const uint32_t qx = quadx[(cx ? S.nq[0][0] : 0) + (int)px], qy = quady[(cy ? S.nq[1][0] : 0) + (int)py];
+  auto prepare = [&](PatchItem<PL>& I, int it, int colour, int fi, uint32_t m, const StepKeys& key) {
+    const uint2 e = table[colour * R.items + it];
+    I.fl = e.x >> 31;
+    if (!I.fl) return;
     // fine order of the quad's block
-    const uint32_t blk = (2u * ((qy >> 24) & 127u) + (uint32_t)cy) * (uint32_t)d.P + 2u * ((qx >> 24) & 127u) + (uint32_t)cx;
-    const uint32_t fcol = ((uint32_t)fo[(m & 1u) * nblk + blk] >> (2 * fi)) & 3u, fx = fcol & 1u, fy = fcol >> 1;
-    const uint32_t kx = ((qx >> 12) & 0xFFFu) + fx, ky = ((qy >> 12) & 0xFFFu) + fy;
-    if ((qx & qy) >> 31) {
-      I.i00 = (int)(((qy & 0xFFFu) + fy) * (uint32_t)pitch + (qx & 0xFFFu) + fx);
-      I.dc = 1;
-      I.dr = pitch;
-    } else {
-      const uint32_t sx = segx[kx], sy = segy[ky];
-      const int c0 = (int)(sx & 0xFFFu), r0 = (int)(sy & 0xFFFu);
-      I.i00 = r0 * pitch + c0;
-      I.dc = (int)((sx >> 12) & 0xFFFu) - c0;
-      I.dr = ((int)((sy >> 12) & 0xFFFu) - r0) * pitch;
-      I.fl |= (sx >> 24) << 1 | (sy >> 24) << 2;
-      if (REFLECT)
-        I.fl |= (ky == 0u ? 16u : 0u) | (ky == GQy - 1u ? 32u : 0u) | (kx == 0u ? 64u : 0u) | (kx == GQ - 1u ? 128u : 0u);
-    }
-    const uint32_t g = ky * GQ + kx;
-    patch_item_draw<PL, LG, REFLECT>(I, key, g, m, rk, S.T, tx, txi);
-    return I;
+    const uint32_t fcol = (uint32_t)fo[(m & 1u) * nblk + (e.y >> 24)] >> (2 * fi), fx = fcol & 1u, fy = (fcol >> 1) & 1u;
+    const uint32_t wide = e.x >> 16, wc = (wide >> fx) & 1u, wr = (wide >> (2u + fy)) & 1u;
+    I.i00 = (int)((e.x & 0xFFFFu) + fx + (fx & wide)) + (fy ? ((wide & 4u) ? 2 * pitch : pitch) : 0);
+    I.dc = 1 + (int)wc - ((fx & (e.x >> 20)) ? R.nsx : 0);   // the last column's right joint is slot 0
+    I.dr = (1 + (int)wr - ((fy & (e.x >> 21)) ? R.nsy : 0)) * pitch;
+    I.fl |= wc << 1 | wr << 2;
+    if (REFLECT)
+      I.fl |= ((e.x >> 23) & (fy ^ 1u) & 1u) << 4 | ((e.x >> 21) & fy) << 5 | ((e.x >> 22) & (fx ^ 1u) & 1u) << 6 |
+              ((e.x >> 20) & fx) << 7;
+    patch_item_draw<PL, LG, REFLECT>(I, key, (e.y & 0xFFFFFFu) + fy * GQ + fx, m, rk, S.T, tx, txi);
   };
 
   auto orders = [&](uint32_t m, int t, int n) {   // the blocks' fine orders of MCS m
@@ -334,7 +331,8 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, RK rk, const Reside
   uint32_t ord = order(m_begin);
   StepKeys key = step_keys(m_begin, rk);
   res_sync(nthr);
-  PatchItem<PL> cur = prepare(tid, order_at(ord, grp >> 2), grp & 3, m_begin, key);
+  PatchItem<PL> cur;
+  prepare(cur, tid, order_at(ord, grp >> 2), grp & 3, m_begin, key);
   bool handed = false;   // the last phase ended with a CTA barrier instead of a hand-over
   uint32_t m = m_begin;
   for (; m < m_end; ++m) {
@@ -349,7 +347,7 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, RK rk, const Reside
       else if (ph > 0 || handed)
         bar_named((uint32_t)(1 + grp), (uint32_t)(2 * gs));
       const int colour = order_at(ord, ph >> 2), fi = ph & 3;
-      const int n = (int)S.col[colour].x;
+      const int n = S.n[colour];
       const int phn = (ph + groups) & 15;   // this group's next phase
       const bool wrap = ph + groups > 15;
       const int colour_n = order_at(wrap ? ord_next : ord, phn >> 2);
@@ -358,9 +356,9 @@ __device__ uint32_t resident_run_patch(const LatticeDesc& d, RK rk, const Reside
         const bool more = it + gs < n;
         if (cur.fl) patch_item_run<PL, LG, REFLECT>(M, pitch, cur, S.T, tx, txi);
         if (groups > 1 && !more && !(joined && ph == 15))
-          bar_arrive((uint32_t)(1 + (grp + 1) % groups), (uint32_t)(2 * gs));
+          bar_arrive((uint32_t)(grp + 1 == groups ? 1 : 2 + grp), (uint32_t)(2 * gs));
         const bool nm = wrap && !more;
-        cur = prepare(more ? it + gs : tid, more ? colour : colour_n, more ? fi : phn & 3, nm ? m + 1u : m,
+        prepare(cur, more ? it + gs : tid, more ? colour : colour_n, more ? fi : phn & 3, nm ? m + 1u : m,
                       nm ? key_next : key);
         if (!more) break;
       }
