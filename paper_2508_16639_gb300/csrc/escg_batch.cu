@@ -488,8 +488,8 @@ __device__ __forceinline__ void batch_patch_chunk(const SlotDesc& sd, SlotState*
   resident_drain<PL>(d, R, dyn);
 }
 
-template <int THREADS>   // 1024 or 512
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) batch_patch_kernel(BatchArgs a, const uint32_t* active) {
+template <int THREADS>   // 640 (one CTA per SM) or 320 (two): 96 registers
+__global__ void __launch_bounds__(THREADS, 640 / THREADS) batch_patch_kernel(BatchArgs a, const uint32_t* active) {
   extern __shared__ __align__(16) uint8_t res_dyn[];
   __shared__ ResidentPatchSmem S;
   __shared__ ResidentLayout R;
@@ -1097,7 +1097,7 @@ cudaError_t launch_batch_kernel(Engine* e, int threads) {
   BatchArgs a{e->d_slots, e->d_states, e->d_ctl, e->d_table, e->log_every, e->spin_limit};
   if (e->tma) {
     BatchTmaArgs ta{a, e->d_maps};
-    const int g = e->grid_tma[tsel(threads)];
+    const int g = e->patch_on ? 1 : e->grid_tma[tsel(threads)];   // 1: nothing in its table, only the chunk to record
     if (threads == 64)
       batch_tma_kernel<64><<<g, 64 + 32, 0, e->stream>>>(ta);
     else if (threads == 128)
@@ -1106,7 +1106,7 @@ cudaError_t launch_batch_kernel(Engine* e, int threads) {
       batch_tma_kernel<256><<<g, 256 + 32, 0, e->stream>>>(ta);
     return cudaGetLastError();
   }
-  const int g = e->grid[tsel(threads)];
+  const int g = e->patch_on ? 1 : e->grid[tsel(threads)];
   if (threads == 64)
     batch_kernel<64><<<g, 64, 0, e->stream>>>(a);
   else if (threads == 128)
@@ -1130,9 +1130,9 @@ cudaError_t launch_resident_kernels(Engine* e) {
 cudaError_t launch_patch(Engine* e) {
   BatchArgs a{e->d_slots, e->d_states, e->d_ctl, e->d_table, e->log_every, e->spin_limit};
   if (e->n_patch <= e->sms)
-    batch_patch_kernel<1024><<<e->n_patch, 1024, e->patch_bytes, e->stream>>>(a, e->d_active);
+    batch_patch_kernel<640><<<e->n_patch, 640, e->patch_bytes, e->stream>>>(a, e->d_active);
   else
-    batch_patch_kernel<512><<<e->n_patch, 512, e->patch_bytes, e->stream>>>(a, e->d_active);
+    batch_patch_kernel<320><<<e->n_patch, 320, e->patch_bytes, e->stream>>>(a, e->d_active);
   return cudaGetLastError();
 }
 
@@ -1221,8 +1221,8 @@ int engine_init(Engine* e, int max_slots, size_t arena_bytes, size_t table_cap, 
     const AxisGeom g = make_axis_geom(L, 2);
     if (slot_axis_ok(g)) e->patch_bytes = std::max(e->patch_bytes, resident_layout(g, 2, L, g, 2, L, 2).bytes);
   }
-  cudaFuncSetAttribute(batch_patch_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, e->patch_bytes);
-  cudaFuncSetAttribute(batch_patch_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, e->patch_bytes);
+  cudaFuncSetAttribute(batch_patch_kernel<320>, cudaFuncAttributeMaxDynamicSharedMemorySize, e->patch_bytes);
+  cudaFuncSetAttribute(batch_patch_kernel<640>, cudaFuncAttributeMaxDynamicSharedMemorySize, e->patch_bytes);
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, e->device);
   e->res_bytes3 = optin - (int)(sizeof(ResidentSmem) + sizeof(SlotDesc)) - 256;
@@ -1483,10 +1483,10 @@ int engine_active(Engine* e, uint32_t* out) {
 
 // Which kernel runs the replicas of kPatchClass.  Resident while no other
 // replica is in the engine and each has half an SM to itself: us per MCS,
-// chunk kernel -> resident, 144 replicas of L = 100, S = 8 43.4 -> 22.7, 138 of
-// L = 64 and 100 42.4 -> 22.8, 8 of them 38.9 -> 22.1; with 518 of them 47.5 -> 58.9,
-// with 576 of L = 100 51.1 -> 64.7, and beside larger replicas, whose visits need
-// the issue slots, 256 of all sizes 74.7 -> 81.0.
+// chunk kernel -> resident, 144 replicas of L = 100, S = 8 43.4 -> 20.7, 138 of
+// L = 64 and 100 42.4 -> 20.6, 264 of them 25.8 (29.7 in CTAs of 512 threads, 64
+// registers); with 518 of them 47.5 -> 58.9, and beside larger replicas, whose
+// visits need the issue slots, 256 of all sizes 74.7 -> 81.0.
 void engine_plan(Engine* e) { e->patch_on = e->n_patch > 0 && e->n_patch == e->n_used && e->n_patch <= 2 * e->sms; }
 
 // Runs up to `chunks` chunks (0: until no replica is active), stopping early
