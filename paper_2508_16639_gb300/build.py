@@ -19,7 +19,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libescg.so")
 SOURCES = ["escg_kernels.cu", "escg_api.cu", "escg_diag.cu", "escg_batch.cu", "escg_noalloc.cu", "escg_owner.cu",
-           "escg_flag.cu"]
+           "escg_flag.cu", "escg_group.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -267,6 +267,8 @@ struct escg {
   double tuned_ms_per_mcs = 0.0;
   int tuned_candidates = 0;      // configurations timed (0: taken from the cache)
   GownConfig gown{};
+  bool use_group = false;        // block owners on macros (reported as use_own or use_gown)
+  GroupConfig group{};
   size_t ob_words = 0;           // boundary-record words allocated (all blocks)
   CUtensorMap tmap{};
   uint32_t spin_limit = kDefaultSpinLimit;
@@ -463,9 +465,10 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   const Partition& p = h->part;
   const Partition& py = h->part_y;
   const int L = h->L, H = h->H;
-  h->use_tma = h->use_ll = h->use_own = h->use_gown = h->use_resident = false;
+  h->use_tma = h->use_ll = h->use_own = h->use_gown = h->use_group = h->use_resident = false;
   h->own_dyn = h->own_threads = 0;
   h->gown = GownConfig{};
+  h->group = GroupConfig{};
   h->use_macro = false;
   h->grid = persistent_grid(h->device, d.uniform64 != 0 && h->bits == 8);
   // the TMA and mailbox kernels are written for square lattices of one byte
@@ -527,6 +530,17 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
       h->gown = cfg;
     }
   }
+  // The owners on macros (escg_group.cu), for the lattices where they beat
+  // the owners above and the flag kernel (group_fn has both sides measured).
+  if (persistent == 5 || (persistent == 1 && (p.P / 2) * (py.P / 2) >= (d.blocks64 ? 9 : 2))) {
+    GroupConfig cfg{};
+    if (persistent_group_config(d, h->device, &cfg, ctas_per_sm) > 0 &&
+        (persistent == 5 || cfg.ctas_per_sm <= kGownDefaultPerSM) && ensure_macros(h)) {
+      if (ensure_records(h, (size_t)p.P * py.P * kGroupRecordWords) != ESCG_OK) return ESCG_ENOMEM;
+      h->use_group = h->use_gown = true;
+      h->group = cfg;
+    }
+  }
   // Whole-lattice residency: on request (4), and by default (1) for a generic
   // partition with 2 x 2 coarse blocks (L, H < 192 and not 128), where it was
   // measured 1.4-2.2x faster than the flag kernel's dependency chain of
@@ -535,7 +549,7 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   if ((persistent == 4 || (persistent == 1 && !d.uniform64 && p.P == 2 && py.P == 2)) &&
       resident_fits(d, h->device)) {
     h->use_resident = true;
-    h->use_gown = false;
+    h->use_own = h->use_gown = h->use_group = false;
   }
   // The flag kernel on a uniform lattice (any bits per site) with more than
   // 4 CTAs per SM requested, or by default (1) with at least kFlag128Ratio times as many
@@ -884,7 +898,7 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
   const uint32_t k = h->opt.log_every;
   // rule variants count log points with the count kernel between launches
   // (the resident kernel and the one on macros count in-kernel for every rule)
-  const bool fused = (h->desc.nbh == 4 && !h->desc.reflect) || h->use_resident || h->use_macro;
+  const bool fused = (h->desc.nbh == 4 && !h->desc.reflect) || h->use_resident || h->use_macro || h->use_group;
   while (h->mcs_enq < target) {
     uint64_t end;
     if (h->opt.persistent && !h->opt.stop_at_extinction && fused) {
@@ -921,6 +935,10 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
       CUDA_TRY(timing_begin(h));
       if (h->use_resident) {
         CUDA_TRY(launch_resident(a, h->stream));
+      } else if (h->use_group) {
+        a.macros = h->d_macros;
+        CUDA_TRY(launch_persistent_group(a, h->group, h->stream));
+        h->launches += 2;   // the array into macros and back
       } else if (h->use_own) {
         CUDA_TRY(launch_persistent_own(a, h->own_dyn, h->own_threads, h->stream));
       } else if (h->use_gown) {
@@ -1249,7 +1267,7 @@ std::map<TuneKey, TuneVal> g_tune;
 // What a selection runs, for dropping candidates that duplicate another.
 std::string kernel_signature(escg* h) {
   char buf[128];
-  snprintf(buf, sizeof buf, "%s/%d/%d/%d/%d", escg_update_kernel(h), h->grid, h->own_threads, h->gown.threads,
+  snprintf(buf, sizeof buf, "%s/%d/%d/%d/%d", escg_update_kernel(h), h->grid, h->own_threads, h->use_group ? h->group.group_threads : h->gown.threads,
            h->flag_threads);
   return buf;
 }

@@ -421,8 +421,21 @@ __global__ void __launch_bounds__(256) macro_drain_kernel(LatticeDesc d, const t
 }
 
 // ---------------------------------------------------------------------------
-size_t macro_bytes(const LatticeDesc& d) {
-  return (size_t)(d.L / 2) * (size_t)(d.H / 2) * (size_t)patch_planes(d);
+cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, cudaStream_t stream) {
+  const dim3 cb(32, 8), cg(((d.L >> 4) + 31) / 32, ((d.H >> 1) + 7) / 8);
+  if (patch_planes(d) == 1)
+    macro_fill_kernel<1><<<cg, cb, 0, stream>>>(d, reinterpret_cast<uint8_t*>(macros));
+  else
+    macro_fill_kernel<2><<<cg, cb, 0, stream>>>(d, reinterpret_cast<uint16_t*>(macros));
+  return cudaGetLastError();
+}
+cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, cudaStream_t stream) {
+  const dim3 cb(32, 8), cg(((d.L >> 4) + 31) / 32, ((d.H >> 1) + 7) / 8);
+  if (patch_planes(d) == 1)
+    macro_drain_kernel<1><<<cg, cb, 0, stream>>>(d, reinterpret_cast<const uint8_t*>(macros));
+  else
+    macro_drain_kernel<2><<<cg, cb, 0, stream>>>(d, reinterpret_cast<const uint16_t*>(macros));
+  return cudaGetLastError();
 }
 
 template <int PL, int NT>
@@ -452,23 +465,12 @@ cudaError_t launch_persistent_macro(const PersistentArgs& args, int grid, cudaSt
   a.rcp_nb = div_rcp32(nb);
   a.rcp_per = div_rcp32(nb >> 2);
   a.rcp_half = div_rcp32((uint32_t)(a.d.P >> 1));
-  const int nt = a.d.L >> 4, rows = a.d.H >> 1;
-  const dim3 cb(32, 8), cg((nt + 31) / 32, (rows + 7) / 8);
-  const bool one = patch_planes(a.d) == 1;
-  if (one)
-    macro_fill_kernel<1><<<cg, cb, 0, stream>>>(a.d, reinterpret_cast<uint8_t*>(a.macros));
-  else
-    macro_fill_kernel<2><<<cg, cb, 0, stream>>>(a.d, reinterpret_cast<uint16_t*>(a.macros));
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_macro_fill(a.d, a.macros, stream);
   if (e != cudaSuccess) return e;
   void* params[] = {&a};
   e = cudaLaunchKernel(macro_kernel_fn(a.d, a.threads), dim3(grid), dim3(a.threads), params, 0, stream);
   if (e != cudaSuccess) return e;
-  if (one)
-    macro_drain_kernel<1><<<cg, cb, 0, stream>>>(a.d, reinterpret_cast<const uint8_t*>(a.macros));
-  else
-    macro_drain_kernel<2><<<cg, cb, 0, stream>>>(a.d, reinterpret_cast<const uint16_t*>(a.macros));
-  return cudaGetLastError();
+  return launch_macro_drain(a.d, a.macros, stream);
 }
 
 }  // namespace escg_impl

@@ -88,7 +88,7 @@ struct PersistentArgs {
   int32_t fuse_counts;     // 1: counts of log points fused into the visits; 0: the host counts
   int32_t threads;         // flag kernel on macros: 128 (two sub-blocks per thread, up to 8
                            // CTAs per SM) or 256 (one)
-  void* macros;            // macro array of the flag kernel on uniform partitions (escg_flag.cu)
+  void* macros;            // macro array (escg_flag.cu, escg_group.cu)
   // div_rcp32 of the ticket decode's divisors (blocks per MCS, blocks per
   // coarse phase, half the blocks per row); filled in by launch_persistent
   uint32_t rcp_nb, rcp_per, rcp_half;
@@ -98,10 +98,17 @@ struct PersistentArgs {
 cudaError_t launch_persistent(const PersistentArgs& a, int grid, cudaStream_t stream);
 // Occupancy-derived grid size of the persistent kernel for a lattice.
 int persistent_grid(int device, bool uniform);
-// The flag kernel on macros (uniform partitions, any rule; escg_flag.cu): the
-// lattice array is turned into a.macros (macro_bytes), run there by CTAs of
-// a.threads and written back.  Grid by occupancy.
+// The macro array of a lattice (escg_patch.cuh): rows of macro_pitch macros.
+// Lattice array <-> macros, for uniform partitions and for any.
+int macro_pitch(const LatticeDesc& d);
 size_t macro_bytes(const LatticeDesc& d);
+cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, cudaStream_t stream);
+cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, cudaStream_t stream);
+cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, cudaStream_t stream);
+cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, cudaStream_t stream);
+// The flag kernel on macros (uniform partitions, any rule; escg_flag.cu): the
+// lattice array is turned into a.macros, run there by CTAs of a.threads and
+// written back.  Grid by occupancy.
 int persistent_macro_grid(const LatticeDesc& d, int device, int threads);
 cudaError_t launch_persistent_macro(const PersistentArgs& a, int grid, cudaStream_t stream);
 
@@ -152,6 +159,24 @@ struct GownArgs {
 // configuration; min_per_sm as for persistent_own_config.
 int persistent_gown_config(const LatticeDesc& d, int device, GownConfig* cfg, int min_per_sm = 0);
 cudaError_t launch_persistent_gown(const PersistentArgs& a, const GownConfig& cfg, cudaStream_t stream);
+// Group owners on macros (escg_group.cu): any partition with fine segments of
+// 2 or 3 sites, every rule and storage.  CTA g owns a 2 x 2 group of blocks for
+// the whole launch with their macros in shared memory and exchanges boundary
+// records (a.ob, kGroupRecordWords per block); a.macros as for the flag
+// kernel.  All (P/2)(Py/2) CTAs must be resident at once:
+// persistent_group_config returns the grid size and the launch configuration,
+// or 0 when this lattice or device cannot run the kernel.  min_per_sm as above.
+constexpr int kGroupRecordWords = 64;
+struct GroupConfig {
+  int dyn_bytes;       // dynamic shared memory: the macros, the quad tables, padding
+  int groups;          // groups of threads that take the fine phases in turn: 1 or 4
+  int group_threads;
+  int ctas_per_sm;
+  int pitch;           // macros per row in shared memory
+  int quads, nq_max;   // the quad tables behind the macros: byte offset, entries per block
+};
+int persistent_group_config(const LatticeDesc& d, int device, GroupConfig* cfg, int min_per_sm = 0);
+cudaError_t launch_persistent_group(const PersistentArgs& a, const GroupConfig& cfg, cudaStream_t stream);
 // Completes the lattice array after a mailbox launch that ended at MCS
 // m_end: every edge cell of a block that a neighbour's visit wrote last (in
 // MCS m_end - 1) takes the value from that neighbour's record.  Does nothing

@@ -437,10 +437,11 @@ struct PatchItem {
 
 // The random words of sub-block g in MCS m and, for a 2 x 2 one, its steps;
 // fl and the macro indexes are set.
-template <int PL, int LG, bool REFLECT, class RK>
+// WIDE = false: every sub-block is 2 x 2.
+template <int PL, int LG, bool REFLECT, bool WIDE = true, class RK>
 __device__ __forceinline__ void patch_item_draw(PatchItem<PL>& I, const StepKeys& key, uint32_t g, uint32_t m,
                                                 RK rk, const PatchTables& T, uint32_t tx, uint32_t txi) {
-  if (!(I.fl & 6u)) {
+  if (!WIDE || !(I.fl & 6u)) {
     I.s = patch_steps2<PL, LG, REFLECT>(philox_step(key, g, rk), T, tx, txi, REFLECT ? I.fl >> 4 : 0u);
   } else {
     // the three calls side by side, also where a 2 x 3 sub-block needs two:
@@ -463,11 +464,11 @@ __device__ __forceinline__ void patch_item_draw(PatchItem<PL>& I, const StepKeys
 }
 
 // All its attempts, from and to its macros.
-template <int PL, int LG, bool REFLECT>
+template <int PL, int LG, bool REFLECT, bool WIDE = true>
 __device__ __forceinline__ void patch_item_run(typename MacroOf<PL>::type* __restrict__ M, int pitch,
                                                const PatchItem<PL>& I, const PatchTables& T, uint32_t tx,
                                                uint32_t txi) {
-  if (!(I.fl & 6u)) {
+  if (!WIDE || !(I.fl & 6u)) {
     uint32_t v[PL];
     patch_load2<PL>(M, I.i00, I.dc, I.dr, v);
     patch_run2<PL>(v, I.s, T);

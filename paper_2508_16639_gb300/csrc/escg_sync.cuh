@@ -38,6 +38,17 @@ __device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t n) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+// The same with a constant id: with an id in a register a CTA reserves all 16
+// barriers, and an SM then holds fewer CTAs.
+template <int ID>
+__device__ __forceinline__ void bar_named(uint32_t n) {
+  asm volatile("bar.sync %0, %1;" ::"n"(ID), "r"(n) : "memory");
+}
+template <int ID>
+__device__ __forceinline__ void bar_arrive(uint32_t n) {
+  asm volatile("bar.arrive %0, %1;" ::"n"(ID), "r"(n) : "memory");
+}
+
 // Writes the log entry of MCS m_end from counts c[0..S]; stasis check.
 static __device__ void write_log_entry(RunState* st, LogBuffers lb, int S, uint32_t m_end, uint32_t log_every,
                                       const unsigned long long* c, int stop_at_extinction) {
