@@ -569,6 +569,11 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
       h->grid = persistent_macro_grid(d, h->device, 128);
     }
   }
+  // The flag kernel on macros, any other partition
+  if (flag && persistent != 0 && !d.blocks64 && persistent_macro_any_grid(d, h->device) > 0 && ensure_macros(h)) {
+    h->use_macro = true;
+    h->grid = persistent_macro_any_grid(d, h->device);
+  }
   if (ctas_per_sm > 0) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);

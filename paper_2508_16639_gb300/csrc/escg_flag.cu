@@ -100,6 +100,22 @@ __device__ __forceinline__ void flag_count(FlagSmem<PL>& sm, int S, int k, int s
   }
 }
 
+// A block's counts are in st->acc[ring]; the last of the nb blocks writes the
+// log entry of MCS m + 1.
+static __device__ __noinline__ void flag_log(RunState* st, const PersistentArgs& a, uint32_t m, uint32_t ring, uint32_t nb) {
+  __threadfence();
+  if (atomicAdd(&st->pend[ring], 1u) != nb - 1u) return;
+  __threadfence();
+  unsigned long long c[kMaxStates], rest = (unsigned long long)a.d.L * (unsigned long long)a.d.H;
+  for (int v = 1; v < kMaxStates; ++v) {
+    c[v] = atomicExch(&st->acc[ring][v], 0ull);
+    rest -= c[v];
+  }
+  c[0] = rest;
+  st->pend[ring] = 0;
+  write_log_entry(st, a.lb, a.d.S, m + 1u, a.log_every, c, a.stop_at_extinction);
+}
+
 // Bound by the colour chain while a phase is one wave (L = 3200: issue active
 // 52 %, 37 executed thread instructions per attempt where the byte tile took
 // 52), by integer issue once phases are several waves deep.  us per MCS of
@@ -300,6 +316,246 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 8 : 4)
 }
 
 // ---------------------------------------------------------------------------
+// The same on any partition of at least 4 blocks a side whose segments have 2 or
+// 3 sites and whose blocks at most 256 quads (escg_patch.cuh).  A tile is the
+// block's slots, staged in whole aligned 16-byte pieces: they carry up to 15
+// macros of the blocks left and right, which go back unchanged -- those blocks
+// are idle during the visit, and a piece never reaches a third block (blocks have
+// 24 slots or more).
+constexpr int kAnySlots = 45;    // of a block along an axis, right joint included: at most 80 sites
+constexpr int kAnyPitch = 80;    // macros per tile row: 16-byte rows; the rows of two quads fall into different banks
+
+template <int PL>
+struct AnySmem {
+  alignas(16) typename MacroOf<PL>::type tile[kAnySlots * kAnyPitch];
+  PatchTables T;
+  uint32_t quads[4][256];   // by wider block along the columns (1), along the rows (2)
+  uint32_t hist[kMaxStates];
+  uint4 dec;
+  uint32_t ord, forder, quit, abort;
+};
+
+// flag_count for a tile of slots 0 .. ncx, 0 .. ncy from column xoff on.  Out of
+// line: its registers must not count against the visit's.
+template <int PL>
+__device__ __noinline__ void any_count(AnySmem<PL>& sm, int xoff, int ncx, int ncy, int S, int k, int sV, int sH, int sD) {
+  constexpr int kPer = 4 / PL;
+  constexpr uint32_t kMacro = PL == 1 ? 0xFFu : 0xFFFFu;
+  const uint32_t* W = reinterpret_cast<const uint32_t*>(sm.tile);
+  const int w0 = xoff / kPer, used = (xoff + ncx) / kPer - w0 + 1;
+  uint32_t cnt[kMaxStates];
+#pragma unroll
+  for (int v = 0; v < kMaxStates; ++v) cnt[v] = 0;
+  for (int i = threadIdx.x; i < (ncy + 1) * used; i += 256) {
+    const int r = i / used, w = w0 + i - r * used;
+    uint32_t x = W[r * (kAnyPitch / kPer) + w], mask = 0;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      const int col = kPer * w + e - xoff;
+      const bool lr = r == 0 || r == ncy, lc = col == 0 || col == ncx;
+      if (col >= 0 && col <= ncx && (!lr || sV < k) && (!lc || sH < k) && (!(lr && lc) || sD < k))
+        mask |= kMacro << (8 * PL * e);
+    }
+    x &= mask;
+#pragma unroll
+    for (int v = 1; v < (PL == 1 ? 4 : kMaxStates); ++v) {
+      if (v > S) break;
+      if (PL == 1) {
+        const uint32_t z = x ^ (uint32_t)(v * 0x55555555u);
+        cnt[v] += __popc(~(z | (z >> 1)) & 0x55555555u);
+      } else {
+        const uint32_t z = x ^ (uint32_t)(v * 0x11111111u), n = z | (z >> 1);
+        cnt[v] += __popc(~(n | (n >> 2)) & 0x11111111u);
+      }
+    }
+  }
+#pragma unroll
+  for (int v = 1; v < (PL == 1 ? 4 : kMaxStates); ++v) {
+    if (v > S) break;
+    const uint32_t s = __reduce_add_sync(0xFFFFFFFFu, cnt[v]);
+    if ((threadIdx.x & 31) == 0 && s) atomicAdd(&sm.hist[v], s);
+  }
+}
+
+// Bound by integer issue where phases are several waves deep, the warps of
+// the leading 3-site segments (9 attempts and three Philox calls each) among it;
+// a phase's words are drawn before the barrier that ends the one before.  us per
+// MCS against the byte tile, 10-MCS counts, M = 1e-4: L = 4800 114.6 -> 90.9 (2.0e11
+// -> 2.5e11 site updates/s), 12700 619 -> 406, Moore 115.1 -> 93.8, reflecting 127.6 ->
+// 110.9, 6400 x 1600 45.9 -> 35.2; at 2 bits per site 193 -> 93.7, at 4 193 -> 118; S = 5,
+// L = 12700 619 -> 478, 8000 287 -> 278, 4800 114.6 -> 115.4 (bytes kept).
+template <int PL, int LG, bool REFLECT>
+__global__ void __launch_bounds__(256, 4) persistent_macro_any_kernel(const __grid_constant__ PersistentArgs a, int nsx,
+                                                                      int nsy, int gp) {
+  typedef typename MacroOf<PL>::type MT;
+  constexpr int kVec = 16 / PL, kLpr = 4 * PL;   // macros per piece, lanes per tile row
+  constexpr int kLoads = (kAnySlots * kLpr + 255) / 256;
+  __shared__ AnySmem<PL> sm;
+  const LatticeDesc& d = a.d;
+  RunState* st = a.st;
+  MT* G = reinterpret_cast<MT*>(a.macros);
+  const int tid = threadIdx.x;
+  const bool run = !ld_volatile(&st->stopped);
+  if (run) {
+    patch_tables_fill<PL>(sm.T, d, tid, 256);
+    for (int i = tid; i < 4 * 256; i += 256) {
+      const bool ax = (i >> 8) & 1, ay = (i >> 9) & 1;
+      const int Qx = ax ? d.ax.Qa : d.ax.Qb, Qy = ay ? d.ay.Qa : d.ay.Qb, q = i & 255;
+      sm.quads[i >> 8][q] = q < (Qx >> 1) * (Qy >> 1)
+                                ? quad_entry(q, Qx >> 1, Qy >> 1, block_wide(d.ax, ax), block_wide(d.ay, ay), kAnyPitch, 0)
+                                : 0xFFFFFFFFu;
+    }
+    const int P = d.P, half = P >> 1, Py = d.Py;
+    const uint32_t nb = (uint32_t)(P * Py), per = nb >> 2;
+    const uint64_t total = (uint64_t)a.n_mcs * nb;
+    const uint32_t GQ = (uint32_t)d.GQ, GQy = (uint32_t)(d.ay.r * d.ay.Qa + (Py - d.ay.r) * d.ay.Qb);
+    // tickets and flags as in persistent_macro_kernel
+    constexpr int kTicketThread = 32;
+    uint32_t c_m = 0xFFFFFFFFu, c_ord = 0, t_next = 0, ab_next = 0;
+    if (tid == kTicketThread) {
+      t_next = atomicAdd(&st->ticket, 1u);
+      ab_next = ld_volatile(&st->abort);
+    }
+    for (;;) {
+      if (tid == kTicketThread) {
+        const uint32_t t = t_next;
+        const uint32_t quit = ((uint64_t)t >= total) || ab_next;
+        if (!quit) {
+          uint32_t rem, j, jx;
+          const uint32_t m = a.m_begin + div_by_rcp(t, nb, a.rcp_nb, rem);
+          if (m != c_m) {
+            c_m = m;
+            c_ord = colour_order(philox10_rk(make_uint4(0u, 0u, m, kTagOrder), d.rk).x, d.perm24);
+          }
+          sm.ord = c_ord;
+          const uint32_t kk = div_by_rcp(rem, per, a.rcp_per, j);
+          const uint32_t jy = div_by_rcp(j, (uint32_t)half, a.rcp_half, jx);
+          const uint32_t col = (uint32_t)order_at(c_ord, (int)kk);
+          sm.dec = make_uint4(m, kk, 2u * jx + (col & 1u), 2u * jy + (col >> 1));
+        }
+        sm.quit = quit;
+        sm.abort = 0;
+      }
+      if (tid < kMaxStates) sm.hist[tid] = 0;
+      __syncthreads();
+      if (sm.quit) break;
+      const uint4 dec = sm.dec;
+      const uint32_t m = dec.x, ord = sm.ord;
+      const int k = (int)dec.y, bx = (int)dec.z, by = (int)dec.w, colour = (bx & 1) | ((by & 1) << 1);
+      if (tid == kTicketThread) sm.forder = fine_order(d, bx, by, m);
+      if (tid < 9) {
+        const int dx = tid % 3 - 1, dy = tid / 3 - 1;
+        const int ncol = colour ^ ((dx & 1) | ((dy & 1) << 1));
+        const uint32_t need = (tid == 4) ? m : (slot_of(ord, ncol) < k ? m + 1u : m);
+        const uint32_t* flag = a.done + wrap(by + dy, Py) * P + wrap(bx + dx, P);
+        uint32_t spins = 0;
+        while (ld_acquire(flag) < need) {
+          if ((spins & 15u) == 15u && ld_volatile(&st->abort)) {
+            sm.abort = 1;
+            break;
+          }
+          if (++spins > a.spin_limit) {
+            atomicOr(&st->error, kErrTimeout);
+            atomicExch(&st->abort, 1u);
+            sm.abort = 1;
+            break;
+          }
+          __nanosleep(64);
+        }
+      }
+      // the block, while the pollers wait
+      const StepKeys key = step_keys(m, d.rk);
+      const int sx0 = block_slot(d.ax, bx), sy0 = block_slot(d.ay, by), ncx = block_slots(d.ax, bx), ncy = block_slots(d.ay, by);
+      const uint32_t f0x = (uint32_t)(min(bx, d.ax.r) * d.ax.Qa + max(bx - d.ax.r, 0) * d.ax.Qb);
+      const uint32_t f0y = (uint32_t)(min(by, d.ay.r) * d.ay.Qa + max(by - d.ay.r, 0) * d.ay.Qb);
+      const uint32_t q = sm.quads[(bx < d.ax.r ? 1 : 0) + (by < d.ay.r ? 2 : 0)][tid];
+      const int p0 = sx0 / kVec, xoff = sx0 - p0 * kVec;
+      const bool wrap_x = sx0 + ncx == nsx;   // the right joint slot is slot 0
+      const int np = (xoff + ncx - (wrap_x ? 1 : 0)) / kVec + 1;
+      __syncthreads();
+      if (sm.abort) break;   // uniform across the CTA
+      uint4 v[kLoads];
+      uint32_t w[kLoads];
+      auto row_at = [&](int i) {
+        const int y = sy0 + i / kLpr;
+        return G + (size_t)(y == nsy ? 0 : y) * gp;
+      };
+#pragma unroll
+      for (int j = 0; j < kLoads; ++j) {
+        const int i = tid + j * 256, p = i % kLpr;
+        if (i / kLpr > ncy || p >= np) continue;
+        const MT* row = row_at(i);
+        v[j] = __ldcg(reinterpret_cast<const uint4*>(row + (p0 + p) * kVec));
+        if (wrap_x && p == np - 1) w[j] = __ldcg(row);
+      }
+      const uint32_t ford = sm.forder;
+      PatchItem<PL> I;
+      auto draw = [&](int fi) {
+        const uint32_t fcol = (ford >> (2 * fi)) & 3u, fx = fcol & 1u, fy = fcol >> 1;
+        const uint32_t wc = (q >> (28u + fx)) & 1u, wr = (q >> (30u + fy)) & 1u;
+        I.i00 = (int)(q & 0xFFFFu) + xoff + (int)fx + (int)(fx & (q >> 28)) + (fy ? kAnyPitch : 0) +
+                (fy & (q >> 30) ? kAnyPitch : 0);
+        I.dc = 1 + (int)wc;
+        I.dr = wr ? 2 * kAnyPitch : kAnyPitch;
+        I.fl = 1u | wc << 1 | wr << 2;
+        const uint32_t kx = f0x + 2u * ((q >> 16) & 63u) + fx, ky = f0y + 2u * ((q >> 22) & 63u) + fy;
+        if (REFLECT)
+          I.fl |= (ky == 0u ? 16u : 0u) | (ky == GQy - 1u ? 32u : 0u) | (kx == 0u ? 64u : 0u) | (kx == GQ - 1u ? 128u : 0u);
+        patch_item_draw<PL, LG, REFLECT>(I, key, ky * GQ + kx, m, d.rk, sm.T, d.tx, d.txi);
+      };
+      const bool item = q != 0xFFFFFFFFu;
+      if (item) draw(0);
+#pragma unroll
+      for (int j = 0; j < kLoads; ++j) {
+        const int i = tid + j * 256, r = i / kLpr, p = i % kLpr;
+        if (r > ncy || p >= np) continue;
+        *reinterpret_cast<uint4*>(sm.tile + r * kAnyPitch + p * kVec) = v[j];
+        if (wrap_x && p == np - 1) sm.tile[r * kAnyPitch + xoff + ncx] = (MT)w[j];
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int fi = 0; fi < 4; ++fi) {
+        if (item) patch_item_run<PL, LG, REFLECT>(sm.tile, kAnyPitch, I, sm.T, d.tx, d.txi);
+        if (item && fi < 3) draw(fi + 1);
+        __syncthreads();
+      }
+      const bool log_point = a.fuse_counts && ((m + 1u) % a.log_every) == 0u;
+      if (log_point)
+        any_count<PL>(sm, xoff, ncx, ncy, d.S, k, slot_of(ord, colour ^ 2), slot_of(ord, colour ^ 1), slot_of(ord, colour ^ 3));
+#pragma unroll
+      for (int j = 0; j < kLoads; ++j) {
+        const int i = tid + j * 256, r = i / kLpr, p = i % kLpr;
+        if (r > ncy || p >= np) continue;
+        MT* row = row_at(i);
+        *reinterpret_cast<uint4*>(row + (p0 + p) * kVec) = *reinterpret_cast<const uint4*>(sm.tile + r * kAnyPitch + p * kVec);
+        if (wrap_x && p == np - 1) row[0] = sm.tile[r * kAnyPitch + xoff + ncx];
+      }
+      __syncthreads();
+      if (tid == 0 && by * P + bx != a.stall_block) st_release(a.done + by * P + bx, m + 1u);
+      if (tid == kTicketThread) {
+        t_next = atomicAdd(&st->ticket, 1u);
+        ab_next = ld_volatile(&st->abort);
+      }
+      if (log_point) {
+        const uint32_t ring = ((m + 1u) / a.log_every) % (uint32_t)kPendRing;
+        if (tid >= 1 && tid <= d.S && sm.hist[tid])
+          atomicAdd(&st->acc[ring][tid], (unsigned long long)sm.hist[tid]);
+        __syncthreads();
+        if (tid == 0) flag_log(st, a, m, ring, nb);
+      }
+    }
+  }
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(&st->exited, 1u) == gridDim.x - 1u) {
+      st->exited = 0;
+      st->ticket = 0;
+      if (!st->stopped && !st->abort) st->mcs = a.m_begin + a.n_mcs;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Lattice array <-> macros.  One thread moves 16 columns of one row slot: the
 // rows 2 ky - 1 and 2 ky (periodic), 8 macros.
 
@@ -450,6 +706,35 @@ static const void* macro_kernel_fn(const LatticeDesc& d, int nt) {
   return nt == 128 ? macro_fn<2, 128>(d) : macro_fn<2, 256>(d);
 }
 
+static const void* macro_any_fn(const LatticeDesc& d) {
+#define ANY_FN(PL, LG, RF) reinterpret_cast<const void*>(&persistent_macro_any_kernel<PL, LG, RF>)
+  if (patch_planes(d) == 1) return d.nbh == 8 ? (d.reflect ? ANY_FN(1, 3, true) : ANY_FN(1, 3, false))
+                                              : (d.reflect ? ANY_FN(1, 2, true) : ANY_FN(1, 2, false));
+  return d.nbh == 8 ? (d.reflect ? ANY_FN(2, 3, true) : ANY_FN(2, 3, false))
+                    : (d.reflect ? ANY_FN(2, 2, true) : ANY_FN(2, 2, false));
+#undef ANY_FN
+}
+
+int persistent_macro_any_grid(const LatticeDesc& d, int device) {
+  if (d.P < 4 || d.Py < 4 || !slot_axis_ok(d.ax) || !slot_axis_ok(d.ay)) return 0;
+  const int Qx = d.ax.r > 0 && d.ax.Qa > d.ax.Qb ? d.ax.Qa : d.ax.Qb, Qy = d.ay.r > 0 && d.ay.Qa > d.ay.Qb ? d.ay.Qa : d.ay.Qb;
+  if ((Qx >> 1) * (Qy >> 1) > 256) return 0;
+  int sms = 0, occ = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, macro_any_fn(d), 256, 0) != cudaSuccess) return 0;
+  const int grid = sms * (occ < 4 ? occ : 4);
+  // Where it beats the flag kernel on bytes: with 2 bits per site (S <= 3), the
+  // reflecting boundary only once a phase is two waves deep (its mirrored steps
+  // lengthen the chain: L = 800, Moore, 44.1 -> 52.5 us per MCS); with 4 bits only
+  // past half of the L2, where the bytes no longer stay.  Packed lattices, whose
+  // byte tiles cost a conversion each way, always.
+  if (d.bits == 8) {
+    const bool deep = (int64_t)d.P * d.Py / 4 >= 2 * (int64_t)grid;
+    if (patch_planes(d) == 1 ? d.reflect && !deep : d.reflect || (size_t)d.H * d.pitch < (64u << 20)) return 0;
+  }
+  return grid;
+}
+
 int persistent_macro_grid(const LatticeDesc& d, int device, int threads) {
   int sms = 0, occ = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
@@ -465,8 +750,15 @@ cudaError_t launch_persistent_macro(const PersistentArgs& args, int grid, cudaSt
   a.rcp_nb = div_rcp32(nb);
   a.rcp_per = div_rcp32(nb >> 2);
   a.rcp_half = div_rcp32((uint32_t)(a.d.P >> 1));
-  cudaError_t e = launch_macro_fill(a.d, a.macros, stream);
+  const bool any = !a.d.blocks64;
+  cudaError_t e = any ? launch_macro_fill_any(a.d, a.macros, stream) : launch_macro_fill(a.d, a.macros, stream);
   if (e != cudaSuccess) return e;
+  if (any) {
+    int nsx = axis_slots(a.d.ax, a.d.P), nsy = axis_slots(a.d.ay, a.d.Py), gp = macro_pitch(a.d);
+    void* params[] = {&a, &nsx, &nsy, &gp};
+    e = cudaLaunchKernel(macro_any_fn(a.d), dim3(grid), dim3(256), params, 0, stream);
+    return e != cudaSuccess ? e : launch_macro_drain_any(a.d, a.macros, stream);
+  }
   void* params[] = {&a};
   e = cudaLaunchKernel(macro_kernel_fn(a.d, a.threads), dim3(grid), dim3(a.threads), params, 0, stream);
   if (e != cudaSuccess) return e;

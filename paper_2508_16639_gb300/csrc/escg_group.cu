@@ -84,15 +84,6 @@ struct GroupArgs {
   int32_t quads, nq_max;   // byte offset of the quad tables in shared memory, entries of each
 };
 
-// First joint slot and its fine segment of block b of an axis.
-__host__ __device__ inline int block_slot(const AxisGeom& g, int b) {
-  const int na = b < g.r ? b : g.r;
-  return na * (g.Qa + block_wide(g, true)) + (b - na) * (g.Qb + block_wide(g, false));
-}
-__host__ __device__ inline int block_slots(const AxisGeom& g, int b) {
-  return b < g.r ? g.Qa + block_wide(g, true) : g.Qb + block_wide(g, false);
-}
-
 __device__ __forceinline__ void group_block(const LatticeDesc& d, int gx, int gy, int c, int pitch, GroupBlock& B) {
   const int cx = c & 1, cy = c >> 1, bx = 2 * gx + cx, by = 2 * gy + cy;
   const BlockSpan X = block_span(d.ax, bx), Y = block_span(d.ay, by);
@@ -111,29 +102,8 @@ __device__ __forceinline__ void group_block(const LatticeDesc& d, int gx, int gy
   B.nq = B.hx * B.hy;
 }
 
-// Quad i of a block, those of 2 x 2 sub-blocks only first (so that warps are
-// of one kind), then the leading rows, then the leading columns: its top
-// left macro (16 bits) | qx << 16 | qy << 22 (6 bits each) | 3-site segments
-// (2 qx, 2 qx + 1 at bits 28, 29; 2 qy, 2 qy + 1 at bits 30, 31).
 __device__ __forceinline__ uint32_t group_quad(const GroupBlock& B, int pitch, int i) {
-  const int ix = (B.frx + 1) >> 1, iy = (B.fry + 1) >> 1, rx = B.hx - ix, nreg = rx * (B.hy - iy), top = B.hx * iy;
-  int qx, qy;
-  if (i < nreg) {
-    qy = i / rx;
-    qx = i - qy * rx + ix;
-    qy += iy;
-  } else if (i < nreg + top) {
-    qy = (i - nreg) / B.hx;
-    qx = i - nreg - qy * B.hx;
-  } else {
-    qy = (i - nreg - top) / ix;
-    qx = i - nreg - top - qy * ix;
-    qy += iy;
-  }
-  const int fx = 2 * qx, fy = 2 * qy;
-  const uint32_t wide = (fx < B.frx ? 1u : 0u) | (fx + 1 < B.frx ? 2u : 0u) | (fy < B.fry ? 4u : 0u) | (fy + 1 < B.fry ? 8u : 0u);
-  return (uint32_t)(B.base + (fy + min(fy, B.fry)) * pitch + fx + min(fx, B.frx)) | ((uint32_t)qx << 16) |
-         ((uint32_t)qy << 22) | (wide << 28);
+  return quad_entry(i, B.hx, B.hy, B.frx, B.fry, pitch, B.base);
 }
 
 // Record word i of block c; false if there is none.
@@ -595,13 +565,21 @@ __device__ __forceinline__ int site_slot(const AxisGeom& g, int ns, int x) {
   return (p & 1) ? 2 * (s + 1 == ns ? 0 : s + 1) : 2 * s + 1;
 }
 
+// A block moves 32 columns (of slots, or of groups of 4 sites) of kConvRows
+// rows: a thread works out its columns once, the block its rows once (the
+// divisions of the closed form cost more than the loads).
+constexpr int kConvRows = 64;
+
 template <int PL>
 __global__ void __launch_bounds__(256)
     macro_fill_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, typename MacroOf<PL>::type* G) {
   typedef typename MacroOf<PL>::type MT;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= nsx || y >= nsy) return;
-  const int2 c = slot_sites(d.ax, d.L, x), r = slot_sites(d.ay, d.H, y);
+  __shared__ int2 rows[kConvRows];
+  const int x = blockIdx.x * 32 + threadIdx.x, y0 = blockIdx.y * kConvRows, t = threadIdx.y * 32 + threadIdx.x;
+  if (t < kConvRows && y0 + t < nsy) rows[t] = slot_sites(d.ay, d.H, y0 + t);
+  __syncthreads();
+  if (x >= nsx) return;
+  const int2 c = slot_sites(d.ax, d.L, x);
   auto site = [&](int row, int col) -> uint32_t {
     if (row < 0 || col < 0) return 0u;
     const uint8_t* p = d.lat + (size_t)row * d.pitch;
@@ -609,31 +587,44 @@ __global__ void __launch_bounds__(256)
     const uint32_t bit = (uint32_t)col * (uint32_t)d.bits;
     return ((uint32_t)p[bit >> 3] >> (bit & 7u)) & ((1u << d.bits) - 1u);
   };
-  G[(size_t)y * gpitch + x] = (MT)(site(r.x, c.x) | (site(r.x, c.y) << (2 * PL)) | (site(r.y, c.x) << (4 * PL)) |
-                                   (site(r.y, c.y) << (6 * PL)));
+#pragma unroll 4
+  for (int k = threadIdx.y; k < kConvRows; k += 8) {
+    if (y0 + k >= nsy) break;
+    const int2 r = rows[k];
+    G[(size_t)(y0 + k) * gpitch + x] = (MT)(site(r.x, c.x) | (site(r.x, c.y) << (2 * PL)) | (site(r.y, c.x) << (4 * PL)) |
+                                            (site(r.y, c.y) << (6 * PL)));
+  }
 }
 
-// One group of 4 sites per thread.
 template <int PL>
 __global__ void __launch_bounds__(256)
     macro_drain_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, const typename MacroOf<PL>::type* G) {
-  const int c0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x), y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (c0 >= d.L || y >= d.H) return;
-  const int my = site_slot(d.ay, nsy, y);
-  const typename MacroOf<PL>::type* row = G + (size_t)(my >> 1) * gpitch;
-  uint32_t u = 0;
+  __shared__ int rows[kConvRows];
+  const int c0 = 4 * (blockIdx.x * 32 + threadIdx.x), y0 = blockIdx.y * kConvRows, t = threadIdx.y * 32 + threadIdx.x;
+  if (t < kConvRows && y0 + t < d.H) rows[t] = site_slot(d.ay, nsy, y0 + t);
+  __syncthreads();
+  if (c0 >= d.L) return;
+  int mx[4];
 #pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (c0 + e < d.L) {
-      const int mx = site_slot(d.ax, nsx, c0 + e);
-      u |= (((uint32_t)row[mx >> 1] >> (2 * PL * (2 * (my & 1) + (mx & 1)))) & (PL == 1 ? 3u : 15u)) << (8 * e);
+  for (int e = 0; e < 4; ++e) mx[e] = c0 + e < d.L ? site_slot(d.ax, nsx, c0 + e) : -1;
+#pragma unroll 4
+  for (int k = threadIdx.y; k < kConvRows; k += 8) {
+    const int y = y0 + k;
+    if (y >= d.H) break;
+    const int my = rows[k];
+    const typename MacroOf<PL>::type* row = G + (size_t)(my >> 1) * gpitch;
+    uint32_t u = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (mx[e] >= 0)
+        u |= (((uint32_t)row[mx[e] >> 1] >> (2 * PL * (2 * (my & 1) + (mx[e] & 1)))) & (PL == 1 ? 3u : 15u)) << (8 * e);
+    uint8_t* out = d.lat + (size_t)y * d.pitch;
+    if (d.bits == 8 && c0 + 4 > d.L) {   // no row padding written
+      for (int e = 0; c0 + e < d.L; ++e) out[c0 + e] = (uint8_t)(u >> (8 * e));
+    } else {
+      store_group(out, c0, d.bits, pack4(u, d.bits));
     }
-  uint8_t* out = d.lat + (size_t)y * d.pitch;
-  if (d.bits == 8 && c0 + 4 > d.L) {   // no row padding written
-    for (int e = 0; c0 + e < d.L; ++e) out[c0 + e] = (uint8_t)(u >> (8 * e));
-    return;
   }
-  store_group(out, c0, d.bits, pack4(u, d.bits));
 }
 
 // ---------------------------------------------------------------------------
@@ -644,7 +635,7 @@ size_t macro_bytes(const LatticeDesc& d) {
 
 cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, cudaStream_t stream) {
   const int nsx = axis_slots(d.ax, d.P), nsy = axis_slots(d.ay, d.Py);
-  const dim3 cb(32, 8), cg((nsx + 31) / 32, (nsy + 7) / 8);
+  const dim3 cb(32, 8), cg((nsx + 31) / 32, (nsy + kConvRows - 1) / kConvRows);
   if (patch_planes(d) == 1)
     macro_fill_any_kernel<1><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<uint8_t*>(macros));
   else
@@ -653,7 +644,7 @@ cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, cudaStream
 }
 cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, cudaStream_t stream) {
   const int nsx = axis_slots(d.ax, d.P), nsy = axis_slots(d.ay, d.Py);
-  const dim3 cb(32, 8), cg(((d.L + 3) / 4 + 31) / 32, (d.H + 7) / 8);
+  const dim3 cb(32, 8), cg(((d.L + 3) / 4 + 31) / 32, (d.H + kConvRows - 1) / kConvRows);
   if (patch_planes(d) == 1)
     macro_drain_any_kernel<1><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<const uint8_t*>(macros));
   else

@@ -110,6 +110,8 @@ cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, cud
 // lattice array is turned into a.macros, run there by CTAs of a.threads and
 // written back.  Grid by occupancy.
 int persistent_macro_grid(const LatticeDesc& d, int device, int threads);
+// The same for other partitions (256 threads): 0 where it cannot run.
+int persistent_macro_any_grid(const LatticeDesc& d, int device);
 cudaError_t launch_persistent_macro(const PersistentArgs& a, int grid, cudaStream_t stream);
 
 // Whole-lattice residency: one CTA runs MCS [m_begin, m_begin + n_mcs) with

@@ -551,4 +551,40 @@ __host__ __device__ inline uint32_t quot_rcp_of(int d) { return d <= 1 ? 0u : 0x
 // overshoots n / d by less than n / 2^32 < 1 / d.
 __device__ __forceinline__ uint32_t quot_rcp(uint32_t n, uint32_t rcp) { return rcp ? __umulhi(n, rcp) : n; }
 
+
+// First joint slot of block b of an axis, and its slots up to the next block's.
+__host__ __device__ inline int block_slot(const AxisGeom& g, int b) {
+  const int na = b < g.r ? b : g.r;
+  return na * (g.Qa + block_wide(g, true)) + (b - na) * (g.Qb + block_wide(g, false));
+}
+__host__ __device__ inline int block_slots(const AxisGeom& g, int b) {
+  return b < g.r ? g.Qa + block_wide(g, true) : g.Qb + block_wide(g, false);
+}
+
+// Quad i of a block of hx x hy quads with frx and fry leading segments of 3
+// sites, those of 2 x 2 sub-blocks only first (so that warps are of one kind),
+// then the leading rows, then the leading columns: its top left macro (base
+// added; 16 bits) | qx << 16 | qy << 22 (6 bits each) | 3-site segments (2 qx, 2 qx + 1
+// at bits 28, 29; 2 qy, 2 qy + 1 at bits 30, 31).
+__device__ __forceinline__ uint32_t quad_entry(int i, int hx, int hy, int frx, int fry, int pitch, int base) {
+  const int ix = (frx + 1) >> 1, iy = (fry + 1) >> 1, rx = hx - ix, nreg = rx * (hy - iy), top = hx * iy;
+  int qx, qy;
+  if (i < nreg) {
+    qy = i / rx;
+    qx = i - qy * rx + ix;
+    qy += iy;
+  } else if (i < nreg + top) {
+    qy = (i - nreg) / hx;
+    qx = i - nreg - qy * hx;
+  } else {
+    qy = (i - nreg - top) / ix;
+    qx = i - nreg - top - qy * ix;
+    qy += iy;
+  }
+  const int fx = 2 * qx, fy = 2 * qy;
+  const uint32_t wide = (fx < frx ? 1u : 0u) | (fx + 1 < frx ? 2u : 0u) | (fy < fry ? 4u : 0u) | (fy + 1 < fry ? 8u : 0u);
+  return (uint32_t)(base + (fy + min(fy, fry)) * pitch + fx + min(fx, frx)) | ((uint32_t)qx << 16) | ((uint32_t)qy << 22) |
+         (wide << 28);
+}
+
 }  // namespace escg_impl
