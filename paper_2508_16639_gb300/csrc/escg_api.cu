@@ -519,7 +519,8 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   // Block owners on a generic partition (von Neumann rule, periodic or
   // reflecting, any bits per site): on request (5), and by default (1) from
   // 2 x 2 groups of blocks while the grid needs at most kGownDefaultPerSM
-  // CTAs per SM.  Needs the device to hold one CTA per group at once.
+  // CTAs per SM.  Needs the device to hold one CTA per group at once.  (Lattices
+  // that the owners on macros run are taken over below.)
   if (!d.uniform64 && d.nbh == 4 &&
       (persistent == 5 || (persistent == 1 && (p.P / 2) * (py.P / 2) >= 2))) {
     GownConfig cfg{};

@@ -1559,10 +1559,10 @@ __global__ void __launch_bounds__(kResThreads) resident_kernel(PersistentArgs a)
 
 // The same on the macro layout (escg_resident_patch.cuh).  Bound by the chain
 // of sixteen fine phases an MCS.  Measured against the one-byte image, us per
-// MCS: L = 64 (S = 3, no movement) 17.7 -> 5.8, 64 18.4 -> 5.7, 100 (S = 5) 32.2
-// -> 16.9, 160 25.7 -> 17.7, 191 (S = 5) 35.9 -> 30.6; on request L = 256 41.6 ->
-// 32.8, 400 142 -> 83.  640 threads keep 96 registers a thread; a phase of L =
-// 64 has 64 sub-blocks, so eight groups of 64 threads take the phases in turn.
+// MCS: L = 64 (S = 3, no movement) 17.7 -> 4.4, 64 18.4 -> 4.9, 100 (S = 8) 32.2
+// -> 16.0, 160 25.7 -> 17.9, 191 (S = 8) 35.9 -> 30.5.  640 threads keep 96 registers
+// a thread; a phase of L = 64 has 64 sub-blocks, so eight groups of 64 threads
+// take the phases in turn.
 constexpr int kResPatchThreads = 640;
 template <int PL, int LG, bool REFLECT>
 __global__ void __launch_bounds__(kResPatchThreads, 1) resident_patch_kernel(const __grid_constant__ PersistentArgs a,
