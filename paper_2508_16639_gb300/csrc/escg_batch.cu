@@ -1243,10 +1243,17 @@ int engine_init(Engine* e, int max_slots, size_t arena_bytes, size_t table_cap, 
   return ESCG_OK;
 }
 
-// Places a replica into `slot`: arena memory, tables, initial lattice and
-// counts; it joins the active set at the next chunk.  ESCG_ENOMEM if the
+int engine_upload(Engine* e);
+
+// Places a replica into `slot`: arena memory now, descriptor, tables, initial
+// lattice and counts with the next engine_upload; it joins the active set at the
+// next chunk.  ESCG_ENOMEM if the
 // arena has no room (nothing is changed then).
 int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int slot) {
+  if (e->up.size() >= 4096) {   // bounds the staging memory (11 MB)
+    const int rc = engine_upload(e);
+    if (rc != ESCG_OK) return rc;
+  }
   size_t off = 0;
   if (!e->arena.alloc(pl.bytes, &off)) {
     set_last_error("device arena full");
