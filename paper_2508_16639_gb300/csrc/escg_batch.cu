@@ -1329,7 +1329,7 @@ int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int s
 // The replicas added since the last call, onto the device: one copy of their
 // descriptors and tables (copies of one run of slots for the tensor maps) and
 // two launches for all, where a set-up of each by itself took 55 us (256
-// replicas of sides 64 to 400: 14.1 -> 1.7 ms).
+// replicas of sides 64 to 400: 14.1 -> 1.7 ms).  Waits for them.
 int engine_upload(Engine* e) {
   const size_t n = e->up.size();
   if (!n) return ESCG_OK;
@@ -1342,7 +1342,6 @@ int engine_upload(Engine* e) {
     err = cudaMalloc(&e->d_up, n * sizeof(SlotUpload));
     if (err == cudaSuccess) e->up_cap = n;
   }
-  // pageable copies: the host buffers are free when the calls return
   if (err == cudaSuccess)
     err = cudaMemcpyAsync(e->d_up, e->up.data(), n * sizeof(SlotUpload), cudaMemcpyHostToDevice, e->stream);
   for (size_t i = 0, k; i < n && err == cudaSuccess; i = k) {
@@ -1360,6 +1359,10 @@ int engine_upload(Engine* e) {
     err = cudaGetLastError();
     e->launches += 2;
   }
+  // a pageable copy may still read the host buffers after its call returned:
+  // they are the next replicas' as soon as they are cleared
+  const cudaError_t done = cudaStreamSynchronize(e->stream);
+  if (err == cudaSuccess) err = done;
   e->up.clear();
   e->up_maps.clear();
   if (err != cudaSuccess) {
