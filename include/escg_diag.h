@@ -3,7 +3,7 @@
  * measurement of the GPU's integer-issue rate (the denominator of the
  * Monte Carlo kernels' roofline; the paper has no counterpart) and a
  * host-controlled stall used to test the bounded device-side waits of the
- * persistent kernel without hanging or faulting the GPU.
+ * persistent kernel without hanging or faulting the GPU, and similar hooks.
  */
 #ifndef ESCG_DIAG_H
 #define ESCG_DIAG_H
@@ -48,6 +48,11 @@ int escg_diag_l2_copy(size_t bytes, int reps, double* gbs);
  * handle refuses to run until escg_restore.  block < 0 clears the hook;
  * spin_limit 0 restores the default limit. */
 int escg_debug_stall_block(escg_t* h, int32_t block, uint32_t spin_limit);
+
+/* Test hook: the next n uploads of a server's admitted runs fail before they
+ * begin (as a failed copy would), so that escg_server_step returns ESCG_ECUDA;
+ * the runs stay admitted and the next step uploads them. */
+int escg_debug_fail_uploads(escg_server_t* s, int32_t n);
 
 /* The autotuner's choice for a handle created with escg_options.autotune:
  * the launch mode (escg_options.persistent) and CTAs per SM it runs with,

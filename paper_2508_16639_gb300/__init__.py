@@ -431,6 +431,10 @@ class Server:
         """Cancel a queued or running run between steps (see escg_server_cancel)."""
         check(load().escg_server_cancel(self._h, int(rid)))
 
+    def debug_fail_uploads(self, n: int):
+        """Test hook: the next n uploads of admitted runs fail."""
+        check(load().escg_debug_fail_uploads(self._h, int(n)))
+
     def poll(self, cap: int = 65536):
         ids = np.zeros(cap, dtype=np.int64)
         n = C.c_int32()

@@ -1065,10 +1065,11 @@ struct Engine {
   CUtensorMap* d_maps = nullptr;  // one TMA tensor map per slot
   bool tma = true;                // warp-specialised TMA chunk kernel
   int grid_tma[3] = {0, 0, 0};
-  std::vector<SlotUpload> up;     // replicas added since the last engine_upload
+  std::vector<SlotUpload> up;     // replicas added and not yet on the device (at most kUpload)
   std::vector<CUtensorMap> up_maps;
   SlotUpload* d_up = nullptr;
-  size_t up_cap = 0;
+  static constexpr size_t kUpload = 4096;   // bounds the staging memory (11 MB)
+  int fail_uploads = 0;           // test hook: uploads that fail before they begin
   bool settled = false;           // no work enqueued since the last engine_check
   uint32_t* h_pinned = nullptr;   // pinned host words (admit list staging, counters)
   size_t table_cap = 0;
@@ -1191,6 +1192,8 @@ int engine_init(Engine* e, int max_slots, size_t arena_bytes, size_t table_cap, 
   if (err == cudaSuccess) err = cudaMalloc(&e->d_table, sizeof(uint32_t) * table_cap);
   if (err == cudaSuccess) err = cudaMalloc(&e->d_admit, sizeof(uint32_t) * (max_slots + 1));
   if (err == cudaSuccess) err = cudaMalloc(&e->d_maps, sizeof(CUtensorMap) * max_slots);
+  if (err == cudaSuccess)
+    err = cudaMalloc(&e->d_up, sizeof(SlotUpload) * std::min<size_t>((size_t)max_slots, Engine::kUpload));
   if (err == cudaSuccess) err = cudaMallocHost(&e->h_pinned, sizeof(uint32_t) * (max_slots + 16));
   if (err == cudaSuccess) err = cudaMemsetAsync(e->d_ctl, 0, sizeof(BatchCtl), e->stream);
   if (err == cudaSuccess) err = cudaMemsetAsync(e->d_states, 0, sizeof(SlotState) * max_slots, e->stream);
@@ -1250,7 +1253,7 @@ int engine_upload(Engine* e);
 // next chunk.  ESCG_ENOMEM if the
 // arena has no room (nothing is changed then).
 int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int slot) {
-  if (e->up.size() >= 4096) {   // bounds the staging memory (11 MB)
+  if (e->up.size() >= Engine::kUpload) {
     const int rc = engine_upload(e);
     if (rc != ESCG_OK) return rc;
   }
@@ -1329,18 +1332,17 @@ int engine_add(Engine* e, const escg_replica_spec& sp, const SlotPlan& pl, int s
 // The replicas added since the last call, onto the device: one copy of their
 // descriptors and tables (copies of one run of slots for the tensor maps) and
 // two launches for all, where a set-up of each by itself took 55 us (256
-// replicas of sides 64 to 400: 14.1 -> 1.7 ms).  Waits for them.
+// replicas of sides 64 to 400: 14.1 -> 1.7 ms).  Waits for them.  After a failure
+// the replicas stay in the list and the next call begins again: what a part of
+// it has placed is placed once more.
 int engine_upload(Engine* e) {
   const size_t n = e->up.size();
   if (!n) return ESCG_OK;
   e->settled = false;
   cudaError_t err = cudaSuccess;
-  if (e->up_cap < n) {
-    cudaFree(e->d_up);   // waits for its last use
-    e->d_up = nullptr;
-    e->up_cap = 0;
-    err = cudaMalloc(&e->d_up, n * sizeof(SlotUpload));
-    if (err == cudaSuccess) e->up_cap = n;
+  if (e->fail_uploads > 0) {
+    e->fail_uploads--;
+    err = cudaErrorMemoryAllocation;
   }
   if (err == cudaSuccess)
     err = cudaMemcpyAsync(e->d_up, e->up.data(), n * sizeof(SlotUpload), cudaMemcpyHostToDevice, e->stream);
@@ -1363,12 +1365,13 @@ int engine_upload(Engine* e) {
   // they are the next replicas' as soon as they are cleared
   const cudaError_t done = cudaStreamSynchronize(e->stream);
   if (err == cudaSuccess) err = done;
-  e->up.clear();
-  e->up_maps.clear();
   if (err != cudaSuccess) {
+    cudaGetLastError();   // the next launch's check must not find it
     set_last_error("replica set-up failed: %s", cudaGetErrorString(err));
     return ESCG_ECUDA;
   }
+  e->up.clear();
+  e->up_maps.clear();
   return ESCG_OK;
 }
 
@@ -1959,6 +1962,15 @@ int escg_server_stats(escg_server_t* s, int32_t* resident, int32_t* queued, uint
   if (resident) *resident = s->resident;
   if (queued) *queued = (int32_t)s->queue.size();
   if (bytes_in_use) *bytes_in_use = s->e.arena.used();
+  return ESCG_OK;
+}
+
+int escg_debug_fail_uploads(escg_server_t* s, int32_t n) {
+  if (!s || n < 0) {
+    set_last_error("bad arguments");
+    return ESCG_EINVAL;
+  }
+  s->e.fail_uploads = n;
   return ESCG_OK;
 }
 

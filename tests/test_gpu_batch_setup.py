@@ -1,4 +1,4 @@
-"""Set-up of a batch's replicas, which go to the device in groups of 4096."""
+"""Set-up of the engine's replicas: in groups of 4096, and again after a failure."""
 import numpy as np
 import pytest
 
@@ -37,3 +37,53 @@ def test_more_replicas_than_one_group():
         assert np.array_equal(counts[i, :sp["S"] + 1], O.counts(o, sp["S"])), i
         assert np.array_equal(b.snapshot(i), o), i
     b.close()
+
+
+def _spec(L, seed, max_mcs):
+    return dict(L=L, S=3, digraph=O.circulant(3, (1,)), rates=(1.0, 1.0, 2.0), seed=seed, p_empty=0.25, max_mcs=max_mcs,
+                stop_at_extinction=False)
+
+
+def _finish(srv, left):
+    done = []
+    for _ in range(200):
+        srv.step()
+        done += srv.poll()
+        if len(done) == left:
+            return done
+    raise AssertionError(done)
+
+
+def _check(srv, rid, sp):
+    mcs, _, counts, lat = srv.result(rid, lattice=True)
+    o, _ = O.replay_run(O.init(sp["L"], 3, 0.25, sp["seed"]), sp["digraph"], *sp["rates"], sp["seed"], sp["max_mcs"])
+    assert mcs == sp["max_mcs"] and np.array_equal(lat, o) and np.array_equal(counts[:4], O.counts(o, 3))
+
+
+@pytest.mark.parametrize("fails", [1, 3])
+def test_a_failed_upload_is_made_good_by_the_next_step(fails):
+    """A step whose upload fails reports it and changes nothing: the admitted runs
+    go up with the next step, into fresh slots and into slots that other runs
+    have left."""
+    srv = E.Server(keep_lattice=True, chunks_per_step=1, max_slots=4)
+    first = [_spec(L, 30 + L, 20) for L in (40, 100, 200)]
+    srv.debug_fail_uploads(fails)
+    ids = [srv.submit(sp) for sp in first]
+    for _ in range(fails):
+        with pytest.raises(E.EscgError):
+            srv.step()
+        assert srv.stats()[:2] == (3, 0)
+    assert sorted(_finish(srv, 3)) == ids
+    for rid, sp in zip(ids, first):
+        _check(srv, rid, sp)
+    second = [_spec(L, 60 + L, 20) for L in (300, 64, 90, 200)]   # three reused slots, one fresh
+    ids = [srv.submit(sp) for sp in second]
+    srv.debug_fail_uploads(fails)
+    for _ in range(fails):
+        with pytest.raises(E.EscgError):
+            srv.step()
+        assert srv.poll() == []
+    assert sorted(_finish(srv, 4)) == ids
+    for rid, sp in zip(ids, second):
+        _check(srv, rid, sp)
+    assert srv.stats() == (0, 0, 0)
