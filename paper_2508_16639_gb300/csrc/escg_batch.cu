@@ -1905,6 +1905,10 @@ int escg_server_cancel(escg_server_t* s, int64_t id) {
   }
   s->results[id] = std::move(res);
   s->finished.push_back(id);
+  // a run that no step has admitted yet (after a failed one): its slot is
+  // another's next, and admitted twice would be stepped by two items at once
+  std::vector<uint32_t>& pend = s->e.pending_admit;
+  pend.erase(std::remove(pend.begin(), pend.end(), (uint32_t)slot), pend.end());
   engine_release(&s->e, slot);
   s->slot_req[slot] = -1;
   s->free_slots.push_back(slot);

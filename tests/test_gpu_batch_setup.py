@@ -87,3 +87,22 @@ def test_a_failed_upload_is_made_good_by_the_next_step(fails):
     for rid, sp in zip(ids, second):
         _check(srv, rid, sp)
     assert srv.stats() == (0, 0, 0)
+
+
+def test_cancel_after_a_failed_step():
+    """A run cancelled between a step that failed and the next one leaves its
+    slot to another run, which is admitted once."""
+    srv = E.Server(keep_lattice=True, chunks_per_step=1, max_slots=2)
+    keep, gone, late = _spec(200, 1, 40), _spec(200, 2, 40), _spec(300, 3, 40)
+    srv.debug_fail_uploads(1)
+    ids = [srv.submit(keep), srv.submit(gone)]
+    with pytest.raises(E.EscgError):
+        srv.step()
+    srv.cancel(ids[1])
+    mcs, ext, counts, lat = srv.result(ids[1], lattice=True)
+    assert mcs == 0 and not ext and np.array_equal(lat, O.init(200, 3, 0.25, 2))
+    assert srv.poll() == [ids[1]]
+    ids[1] = srv.submit(late)
+    assert sorted(_finish(srv, 2)) == ids
+    _check(srv, ids[0], keep)
+    _check(srv, ids[1], late)
