@@ -431,7 +431,10 @@ void free_handle(escg* h) {
   delete h;
 }
 
-// Boundary records of at least `words` words (zeroed by the next reset).
+// Boundary records of at least `words` words.  New ones are zeroed: no wait
+// takes epoch 0, but what the memory held before may be any epoch, and a
+// selection after creation (the autotuner's cached choice) is followed by no
+// reset.
 int ensure_records(escg* h, size_t words) {
   if (h->ob_words >= words) return ESCG_OK;
   cudaFree(h->d_ob);
@@ -442,6 +445,7 @@ int ensure_records(escg* h, size_t words) {
     return ESCG_ENOMEM;
   }
   h->ob_words = words;
+  CUDA_TRY(cudaMemsetAsync(h->d_ob, 0, words * sizeof(unsigned long long), h->stream));
   return ESCG_OK;
 }
 
