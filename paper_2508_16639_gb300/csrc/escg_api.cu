@@ -1252,17 +1252,18 @@ void escg_destroy(escg_t* h) { free_handle(h); }
 // ---------------------------------------------------------------------------
 // Autotuner.  Every launch mode and CTA count gives the same lattice, so the
 // fastest is a measured, result-neutral choice.  On the first handle of a
-// (device, L, H, S, bits per site, rule) the candidates are timed on a
+// (device, L, H, S, bits per site, rule, certain edges or not) the candidates are timed on a
 // scratch copy of the initial lattice -- 10 MCS to warm up, then 20 MCS
 // between two CUDA events -- and the winner is cached for the process; the
 // handle then starts from its initial lattice at MCS 0 as if just created.
 namespace {
 
 struct TuneKey {
-  int dev, L, H, S, bits, nbh, reflect;
+  int dev, L, H, S, bits, nbh, reflect, planes;   // planes: macros of certain edges take other kernels
   bool operator<(const TuneKey& o) const {
-    const int a[7] = {dev, L, H, S, bits, nbh, reflect}, b[7] = {o.dev, o.L, o.H, o.S, o.bits, o.nbh, o.reflect};
-    for (int i = 0; i < 7; ++i)
+    const int a[8] = {dev, L, H, S, bits, nbh, reflect, planes};
+    const int b[8] = {o.dev, o.L, o.H, o.S, o.bits, o.nbh, o.reflect, o.planes};
+    for (int i = 0; i < 8; ++i)
       if (a[i] != b[i]) return a[i] < b[i];
     return false;
   }
@@ -1307,7 +1308,8 @@ int tune_time(escg* h, const uint8_t* scratch, size_t nbytes, double* ms) {
 }  // namespace
 
 static int autotune(escg* h) {
-  const TuneKey key{h->device, h->L, h->H, h->S, h->bits, h->desc.nbh, h->desc.reflect};
+  const TuneKey key{h->device, h->L, h->H, h->S, h->bits, h->desc.nbh, h->desc.reflect,
+                    h->desc.S <= 3 && h->desc.certain ? 1 : 2};
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find(key);
   if (it != g_tune.end()) {

@@ -44,3 +44,14 @@ def test_cached_choice_starts_on_empty_records(L, S, kw):
         o, _ = O.replay_run(O.init(L, S, 0.2, seed), D, 1.0, 1.0, 2.0, seed, 3, **rule)
         assert np.array_equal(g.snapshot(), o)
         g.close()
+
+
+def test_uncertain_edges_are_tuned_for_themselves():
+    """Certain and uncertain edges run different kernels in the same mode, so
+    neither takes the other's timing."""
+    D = O.circulant(3, (1,))
+    for prob in (None, 0.5 * D):
+        for again in (False, True):
+            g = E.Lattice(400, 3, D, (1.0, 1.0, 2.0), 9, p_empty=0.2, autotune=True, dominance_prob=prob)
+            assert (g.autotune_result[3] == 0) == again
+            g.close()
