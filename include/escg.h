@@ -329,8 +329,9 @@ int32_t escg_batch_active(escg_batch_t* b);
 /* Copies replica i's lattice (L*L bytes) to host memory.  Synchronises. */
 int escg_batch_snapshot(escg_batch_t* b, int32_t i, uint8_t* host_out);
 
-/* CTA size in use (after autotuning: the first chunks time the chunk kernel
- * at 64, 128 and 256 threads, TMA-staged and plain, and keep the fastest),
+/* CTA size of the chunk kernel (after autotuning: the first chunks that it
+ * runs time it at 64, 128 and 256 threads, TMA-staged and plain, and keep the
+ * fastest; 0 before, and for good where every replica stays resident),
  * whether the TMA-staged chunk kernel is in use, and kernel launches so far. */
 int32_t escg_batch_threads(escg_batch_t* b);
 int32_t escg_batch_uses_tma(escg_batch_t* b);

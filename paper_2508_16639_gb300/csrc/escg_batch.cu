@@ -1050,7 +1050,7 @@ struct Engine {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   uint32_t log_every = 10;
-  int threads = 0;          // CTA size in use (0: autotune on the first chunks)
+  int threads = 0;          // CTA size of the chunk kernel (0: autotune on the first chunks it runs)
   bool use_graph = true;
   int max_slots = 0;
   uint8_t* arena_mem = nullptr;
@@ -1512,7 +1512,9 @@ int engine_run(Engine* e, uint64_t chunks, bool until_idle) {
   e->settled = false;
   engine_plan(e);
   uint64_t left = chunks;
-  if (e->threads == 0) {
+  // a chunk that batch_patch_kernel runs times nothing of the chunk kernel,
+  // which then only records it (256 threads while untuned)
+  if (e->threads == 0 && !e->patch_on) {
     rc = engine_autotune(e, &left);
     if (rc != ESCG_OK) return rc;
   }

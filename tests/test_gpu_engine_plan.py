@@ -1,0 +1,52 @@
+"""What the batch engine decides between steps: when it tunes the chunk kernel
+and when it builds its graph.  Lattices are the replay oracle's throughout."""
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_2508_16639_gb300 as E
+from paper_2508_16639_gb300.build import build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build()
+
+
+def _spec(L, seed, max_mcs, S=3, stop=False, X=2.0, p_empty=0.25):
+    return dict(L=L, S=S, digraph=O.circulant(S, (1,) if S == 3 else (1, 2)), rates=(1.0, 1.0, X), seed=seed,
+                p_empty=p_empty, max_mcs=max_mcs, stop_at_extinction=stop)
+
+
+def _check(srv, rid, sp):
+    mcs, _, counts, lat = srv.result(rid, lattice=True)
+    o, _ = O.replay_run(O.init(sp["L"], sp["S"], sp["p_empty"], sp["seed"]), sp["digraph"], *sp["rates"], sp["seed"],
+                        sp["max_mcs"])
+    assert mcs == sp["max_mcs"] and np.array_equal(lat, o)
+
+
+def test_the_chunk_kernel_is_tuned_when_it_runs():
+    """A server whose first steps hold small replicas only keeps the choice of the
+    chunk kernel's CTA size open until a step runs that kernel."""
+    srv = E.Server(keep_lattice=True)
+    specs = [_spec(100, 1, 400), _spec(64, 2, 400, S=5)]
+    ids = [srv.submit(sp) for sp in specs]
+    srv.step()
+    srv.step()
+    assert srv.threads == 0
+    specs.append(_spec(300, 3, 120))
+    ids.append(srv.submit(specs[-1]))
+    srv.step()
+    chosen = (srv.threads, srv.uses_tma)
+    assert chosen[0] in (64, 128, 256)
+    done = set()
+    for _ in range(60):
+        srv.step()
+        done.update(srv.poll())
+        if len(done) == 3:
+            break
+    assert (srv.threads, srv.uses_tma) == chosen
+    for rid, sp in zip(ids, specs):
+        _check(srv, rid, sp)
