@@ -54,6 +54,9 @@ int escg_debug_stall_block(escg_t* h, int32_t block, uint32_t spin_limit);
  * the runs stay admitted and the next step uploads them. */
 int escg_debug_fail_uploads(escg_server_t* s, int32_t n);
 
+/* CUDA graphs that a server has captured and instantiated. */
+int32_t escg_debug_graph_builds(escg_server_t* s);
+
 /* The autotuner's choice for a handle created with escg_options.autotune:
  * the launch mode (escg_options.persistent) and CTAs per SM it runs with,
  * the winner's device time per MCS, and how many distinct configurations

@@ -431,6 +431,10 @@ class Server:
         """Cancel a queued or running run between steps (see escg_server_cancel)."""
         check(load().escg_server_cancel(self._h, int(rid)))
 
+    @property
+    def graph_builds(self) -> int:
+        return int(load().escg_debug_graph_builds(self._h))
+
     def debug_fail_uploads(self, n: int):
         """Test hook: the next n uploads of admitted runs fail."""
         check(load().escg_debug_fail_uploads(self._h, int(n)))

@@ -1086,8 +1086,8 @@ struct Engine {
   int sms = 0;
   bool patch_on = false;          // batch_patch_kernel runs the replicas of kPatchClass
   uint64_t launches = 0;
-  cudaGraphExec_t graph = nullptr;
-  int graph_patch = 0;            // replicas batch_patch_kernel runs in it
+  cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};   // of kGraphChunks chunks, by patch_grid
+  int graph_builds = 0;
   uint32_t spin_limit = 2000000;
   static constexpr int kGraphChunks = 16;
 };
@@ -1128,12 +1128,17 @@ cudaError_t launch_resident_kernels(Engine* e) {
   return cudaGetLastError();
 }
 
+// batch_patch_kernel's CTAs per SM (0: it does not run).  CTAs without a replica
+// leave at once, so that a launch, and a graph of them, does not depend on the
+// number of replicas.
+int patch_grid(const Engine* e) { return !e->patch_on ? 0 : (e->n_patch <= e->sms ? 1 : 2); }
+
 cudaError_t launch_patch(Engine* e) {
   BatchArgs a{e->d_slots, e->d_states, e->d_ctl, e->d_table, e->log_every, e->spin_limit};
-  if (e->n_patch <= e->sms)
-    batch_patch_kernel<640><<<e->n_patch, 640, e->patch_bytes, e->stream>>>(a, e->d_active);
+  if (patch_grid(e) == 1)
+    batch_patch_kernel<640><<<e->sms, 640, e->patch_bytes, e->stream>>>(a, e->d_active);
   else
-    batch_patch_kernel<320><<<e->n_patch, 320, e->patch_bytes, e->stream>>>(a, e->d_active);
+    batch_patch_kernel<320><<<2 * e->sms, 320, e->patch_bytes, e->stream>>>(a, e->d_active);
   return cudaGetLastError();
 }
 
@@ -1146,7 +1151,8 @@ cudaError_t launch_compact(Engine* e) {
 
 void engine_free(Engine* e) {
   if (e->stream) cudaStreamSynchronize(e->stream);
-  if (e->graph) cudaGraphExecDestroy(e->graph);
+  for (cudaGraphExec_t g : e->graph)
+    if (g) cudaGraphExecDestroy(g);
   cudaFree(e->arena_mem);
   cudaFree(e->d_slots);
   cudaFree(e->d_states);
@@ -1455,15 +1461,10 @@ int engine_autotune(Engine* e, uint64_t* chunks_left) {
   return ESCG_OK;
 }
 
+// The graph of the present plan, built the first time a run can launch it.
 int engine_build_graph(Engine* e) {
-  // a graph holds the launches of batch_patch_kernel as they were planned
-  const int patch = e->patch_on ? e->n_patch : 0;
-  if (e->graph && patch != e->graph_patch) {
-    cudaGraphExecDestroy(e->graph);
-    e->graph = nullptr;
-  }
-  if (!e->use_graph || e->graph) return ESCG_OK;
-  e->graph_patch = patch;
+  cudaGraphExec_t& exec = e->graph[patch_grid(e)];
+  if (exec) return ESCG_OK;
   cudaGraph_t g;
   if (cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     set_last_error("CUDA graph capture failed to start");
@@ -1475,11 +1476,13 @@ int engine_build_graph(Engine* e) {
     launch_resident_kernels(e);
     launch_batch_kernel(e, e->threads);
   }
-  if (cudaStreamEndCapture(e->stream, &g) != cudaSuccess || cudaGraphInstantiate(&e->graph, g, 0) != cudaSuccess) {
+  if (cudaStreamEndCapture(e->stream, &g) != cudaSuccess || cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) {
+    exec = nullptr;
     set_last_error("CUDA graph capture failed");
     return ESCG_ECUDA;
   }
   cudaGraphDestroy(g);
+  e->graph_builds++;
   return ESCG_OK;
 }
 
@@ -1518,17 +1521,17 @@ int engine_run(Engine* e, uint64_t chunks, bool until_idle) {
     rc = engine_autotune(e, &left);
     if (rc != ESCG_OK) return rc;
   }
-  rc = engine_build_graph(e);
-  if (rc != ESCG_OK) return rc;
   const uint64_t G = Engine::kGraphChunks;
   while (until_idle || left > 0) {
     bool group = false;
-    if (e->graph && (until_idle || left >= G)) {
-      if (cudaGraphLaunch(e->graph, e->stream) != cudaSuccess) {
+    if (e->use_graph && (until_idle || left >= G)) {
+      rc = engine_build_graph(e);
+      if (rc != ESCG_OK) return rc;
+      if (cudaGraphLaunch(e->graph[patch_grid(e)], e->stream) != cudaSuccess) {
         set_last_error("graph launch failed");
         return ESCG_ECUDA;
       }
-      e->launches += ((e->resident ? 5 : 2) + (e->graph_patch ? 1 : 0)) * G;
+      e->launches += ((e->resident ? 5 : 2) + (e->patch_on ? 1 : 0)) * G;
       left = left >= G ? left - G : 0;
       group = true;
     } else {
@@ -1979,6 +1982,8 @@ int escg_debug_fail_uploads(escg_server_t* s, int32_t n) {
   s->e.fail_uploads = n;
   return ESCG_OK;
 }
+
+int32_t escg_debug_graph_builds(escg_server_t* s) { return s ? s->e.graph_builds : 0; }
 
 int32_t escg_server_threads(escg_server_t* s) { return s ? s->e.threads : 0; }
 int32_t escg_server_uses_tma(escg_server_t* s) { return s ? (int32_t)s->e.tma : 0; }

@@ -50,3 +50,25 @@ def test_the_chunk_kernel_is_tuned_when_it_runs():
     assert (srv.threads, srv.uses_tma) == chosen
     for rid, sp in zip(ids, specs):
         _check(srv, rid, sp)
+
+
+@pytest.mark.parametrize("chunks,builds", [(4, 0), (20, 2)])
+def test_graphs_are_built_once(chunks, builds):
+    """Steps too short for a graph build none; longer ones build one for each
+    kernel they run, however many runs come and go."""
+    srv = E.Server(keep_lattice=True, chunks_per_step=chunks, log_every=2)
+    specs = [_spec(100 if i != 6 else 200, 50 + i, 60 + 90 * i) for i in range(9)]
+    ids, done = [], set()
+    for sp in specs:                      # one more each step, one retired every few
+        ids.append(srv.submit(sp))
+        srv.step()
+        done.update(srv.poll())
+    for _ in range(400):
+        if len(done) == len(ids):
+            break
+        srv.step()
+        done.update(srv.poll())
+    assert done == set(ids)
+    assert srv.graph_builds == builds
+    for rid, sp in zip(ids, specs):
+        _check(srv, rid, sp)
