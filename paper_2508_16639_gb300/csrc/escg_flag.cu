@@ -585,7 +585,8 @@ __device__ __forceinline__ uint32_t macro_unpack4(uint32_t v) {
 }
 
 template <int PL>
-__global__ void __launch_bounds__(256) macro_fill_kernel(LatticeDesc d, typename MacroOf<PL>::type* G) {
+__global__ void __launch_bounds__(256) macro_fill_kernel(LatticeDesc d, typename MacroOf<PL>::type* G, RunState* st) {
+  if (macro_fill_off(st)) return;
   const int nt = d.L >> 4, rows = d.H >> 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x, ky = blockIdx.y * blockDim.y + threadIdx.y;
   if (t >= nt || ky >= rows) return;
@@ -625,7 +626,9 @@ __global__ void __launch_bounds__(256) macro_fill_kernel(LatticeDesc d, typename
 }
 
 template <int PL>
-__global__ void __launch_bounds__(256) macro_drain_kernel(LatticeDesc d, const typename MacroOf<PL>::type* G) {
+__global__ void __launch_bounds__(256) macro_drain_kernel(LatticeDesc d, const typename MacroOf<PL>::type* G,
+                                                         const RunState* st) {
+  if (!st->on_macros) return;
   const int nt = d.L >> 4, rows = d.H >> 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x, ky = blockIdx.y * blockDim.y + threadIdx.y;
   if (t >= nt || ky >= rows) return;
@@ -677,20 +680,20 @@ __global__ void __launch_bounds__(256) macro_drain_kernel(LatticeDesc d, const t
 }
 
 // ---------------------------------------------------------------------------
-cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, cudaStream_t stream) {
+cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, RunState* st, cudaStream_t stream) {
   const dim3 cb(32, 8), cg(((d.L >> 4) + 31) / 32, ((d.H >> 1) + 7) / 8);
   if (patch_planes(d) == 1)
-    macro_fill_kernel<1><<<cg, cb, 0, stream>>>(d, reinterpret_cast<uint8_t*>(macros));
+    macro_fill_kernel<1><<<cg, cb, 0, stream>>>(d, reinterpret_cast<uint8_t*>(macros), st);
   else
-    macro_fill_kernel<2><<<cg, cb, 0, stream>>>(d, reinterpret_cast<uint16_t*>(macros));
+    macro_fill_kernel<2><<<cg, cb, 0, stream>>>(d, reinterpret_cast<uint16_t*>(macros), st);
   return cudaGetLastError();
 }
-cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, cudaStream_t stream) {
+cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, const RunState* st, cudaStream_t stream) {
   const dim3 cb(32, 8), cg(((d.L >> 4) + 31) / 32, ((d.H >> 1) + 7) / 8);
   if (patch_planes(d) == 1)
-    macro_drain_kernel<1><<<cg, cb, 0, stream>>>(d, reinterpret_cast<const uint8_t*>(macros));
+    macro_drain_kernel<1><<<cg, cb, 0, stream>>>(d, reinterpret_cast<const uint8_t*>(macros), st);
   else
-    macro_drain_kernel<2><<<cg, cb, 0, stream>>>(d, reinterpret_cast<const uint16_t*>(macros));
+    macro_drain_kernel<2><<<cg, cb, 0, stream>>>(d, reinterpret_cast<const uint16_t*>(macros), st);
   return cudaGetLastError();
 }
 
@@ -751,18 +754,19 @@ cudaError_t launch_persistent_macro(const PersistentArgs& args, int grid, cudaSt
   a.rcp_per = div_rcp32(nb >> 2);
   a.rcp_half = div_rcp32((uint32_t)(a.d.P >> 1));
   const bool any = !a.d.blocks64;
-  cudaError_t e = any ? launch_macro_fill_any(a.d, a.macros, stream) : launch_macro_fill(a.d, a.macros, stream);
+  cudaError_t e = any ? launch_macro_fill_any(a.d, a.macros, a.st, stream)
+                      : launch_macro_fill(a.d, a.macros, a.st, stream);
   if (e != cudaSuccess) return e;
   if (any) {
     int nsx = axis_slots(a.d.ax, a.d.P), nsy = axis_slots(a.d.ay, a.d.Py), gp = macro_pitch(a.d);
     void* params[] = {&a, &nsx, &nsy, &gp};
     e = cudaLaunchKernel(macro_any_fn(a.d), dim3(grid), dim3(256), params, 0, stream);
-    return e != cudaSuccess ? e : launch_macro_drain_any(a.d, a.macros, stream);
+    return e != cudaSuccess ? e : launch_macro_drain_any(a.d, a.macros, a.st, stream);
   }
   void* params[] = {&a};
   e = cudaLaunchKernel(macro_kernel_fn(a.d, a.threads), dim3(grid), dim3(a.threads), params, 0, stream);
   if (e != cudaSuccess) return e;
-  return launch_macro_drain(a.d, a.macros, stream);
+  return launch_macro_drain(a.d, a.macros, a.st, stream);
 }
 
 }  // namespace escg_impl

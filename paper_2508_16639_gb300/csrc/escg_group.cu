@@ -572,7 +572,8 @@ constexpr int kConvRows = 64;
 
 template <int PL>
 __global__ void __launch_bounds__(256)
-    macro_fill_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, typename MacroOf<PL>::type* G) {
+    macro_fill_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, typename MacroOf<PL>::type* G, RunState* st) {
+  if (macro_fill_off(st)) return;
   typedef typename MacroOf<PL>::type MT;
   __shared__ int2 rows[kConvRows];
   const int x = blockIdx.x * 32 + threadIdx.x, y0 = blockIdx.y * kConvRows, t = threadIdx.y * 32 + threadIdx.x;
@@ -598,7 +599,9 @@ __global__ void __launch_bounds__(256)
 
 template <int PL>
 __global__ void __launch_bounds__(256)
-    macro_drain_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, const typename MacroOf<PL>::type* G) {
+    macro_drain_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, const typename MacroOf<PL>::type* G,
+                           const RunState* st) {
+  if (!st->on_macros) return;
   __shared__ int rows[kConvRows];
   const int c0 = 4 * (blockIdx.x * 32 + threadIdx.x), y0 = blockIdx.y * kConvRows, t = threadIdx.y * 32 + threadIdx.x;
   if (t < kConvRows && y0 + t < d.H) rows[t] = site_slot(d.ay, nsy, y0 + t);
@@ -633,23 +636,23 @@ size_t macro_bytes(const LatticeDesc& d) {
   return (size_t)macro_pitch(d) * (size_t)axis_slots(d.ay, d.Py) * (size_t)patch_planes(d);
 }
 
-cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, cudaStream_t stream) {
+cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, RunState* st, cudaStream_t stream) {
   const int nsx = axis_slots(d.ax, d.P), nsy = axis_slots(d.ay, d.Py);
   const dim3 cb(32, 8), cg((nsx + 31) / 32, (nsy + kConvRows - 1) / kConvRows);
   if (patch_planes(d) == 1)
-    macro_fill_any_kernel<1><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<uint8_t*>(macros));
+    macro_fill_any_kernel<1><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<uint8_t*>(macros), st);
   else
-    macro_fill_any_kernel<2><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<uint16_t*>(macros));
+    macro_fill_any_kernel<2><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<uint16_t*>(macros), st);
   return cudaGetLastError();
 }
-cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, cudaStream_t stream) {
+cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, const RunState* st, cudaStream_t stream) {
   const int nsx = axis_slots(d.ax, d.P), nsy = axis_slots(d.ay, d.Py);
   const dim3 cb(32, 8), cg(((d.L + 3) / 4 + 31) / 32, (d.H + kConvRows - 1) / kConvRows);
   if (patch_planes(d) == 1)
-    macro_drain_any_kernel<1><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<const uint8_t*>(macros));
+    macro_drain_any_kernel<1><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d), reinterpret_cast<const uint8_t*>(macros), st);
   else
     macro_drain_any_kernel<2><<<cg, cb, 0, stream>>>(d, nsx, nsy, macro_pitch(d),
-                                                     reinterpret_cast<const uint16_t*>(macros));
+                                                     reinterpret_cast<const uint16_t*>(macros), st);
   return cudaGetLastError();
 }
 
@@ -760,13 +763,15 @@ cudaError_t launch_persistent_group(const PersistentArgs& a, const GroupConfig& 
   arg.gqy = fine_rows(a.d);
   arg.nsx = axis_slots(a.d.ax, a.d.P);
   arg.nsy = axis_slots(a.d.ay, a.d.Py);
-  cudaError_t e = a.d.blocks64 ? launch_macro_fill(a.d, a.macros, stream) : launch_macro_fill_any(a.d, a.macros, stream);
+  cudaError_t e = a.d.blocks64 ? launch_macro_fill(a.d, a.macros, a.st, stream)
+                                  : launch_macro_fill_any(a.d, a.macros, a.st, stream);
   if (e != cudaSuccess) return e;
   void* params[] = {&arg};
   e = cudaLaunchCooperativeKernel(group_fn(a.d, cfg.groups), dim3((a.d.P / 2) * (a.d.Py / 2)), dim3(cfg.groups * cfg.group_threads),
                                   params, (size_t)cfg.dyn_bytes, stream);
   if (e != cudaSuccess) return e;
-  return a.d.blocks64 ? launch_macro_drain(a.d, a.macros, stream) : launch_macro_drain_any(a.d, a.macros, stream);
+  return a.d.blocks64 ? launch_macro_drain(a.d, a.macros, a.st, stream)
+                      : launch_macro_drain_any(a.d, a.macros, a.st, stream);
 }
 
 }  // namespace escg_impl

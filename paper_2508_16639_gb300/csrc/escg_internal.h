@@ -26,6 +26,7 @@ struct RunState {
   unsigned long long cur[kMaxStates];             // counts being accumulated
   unsigned long long acc[kPendRing][kMaxStates];  // open log points (fused counts)
   uint32_t pend[kPendRing];                       // blocks done per open log point
+  uint32_t on_macros;  // the last fill of the macro array took the lattice (it does not while stopped)
 };
 
 constexpr uint32_t kErrTimeout = 1u;
@@ -99,13 +100,14 @@ cudaError_t launch_persistent(const PersistentArgs& a, int grid, cudaStream_t st
 // Occupancy-derived grid size of the persistent kernel for a lattice.
 int persistent_grid(int device, bool uniform);
 // The macro array of a lattice (escg_patch.cuh): rows of macro_pitch macros.
-// Lattice array <-> macros, for uniform partitions and for any.
+// Lattice array <-> macros, for uniform partitions and for any.  A stopped
+// lattice is left alone: it may hold values that no macro does.
 int macro_pitch(const LatticeDesc& d);
 size_t macro_bytes(const LatticeDesc& d);
-cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, cudaStream_t stream);
-cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, cudaStream_t stream);
-cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, cudaStream_t stream);
-cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, cudaStream_t stream);
+cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, RunState* st, cudaStream_t stream);
+cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, const RunState* st, cudaStream_t stream);
+cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, RunState* st, cudaStream_t stream);
+cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, const RunState* st, cudaStream_t stream);
 // The flag kernel on macros (uniform partitions, any rule; escg_flag.cu): the
 // lattice array is turned into a.macros, run there by CTAs of a.threads and
 // written back.  Grid by occupancy.

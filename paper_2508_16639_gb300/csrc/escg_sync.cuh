@@ -49,6 +49,14 @@ __device__ __forceinline__ void bar_arrive(uint32_t n) {
   asm volatile("bar.arrive %0, %1;" ::"n"(ID), "r"(n) : "memory");
 }
 
+// Whether a fill of the macro array has to leave a stopped lattice alone, which
+// the drain then does too.  Called by every thread of a fill.
+__device__ __forceinline__ bool macro_fill_off(RunState* st) {
+  const bool off = st->stopped != 0u;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) st->on_macros = off ? 0u : 1u;
+  return off;
+}
+
 // Writes the log entry of MCS m_end from counts c[0..S]; stasis check.
 static __device__ void write_log_entry(RunState* st, LogBuffers lb, int S, uint32_t m_end, uint32_t log_every,
                                       const unsigned long long* c, int stop_at_extinction) {
