@@ -3,11 +3,11 @@
 // bits per site.
 //
 // persistent_kernel's work items and flags (escg_kernels.cu), on the layout
-// of escg_patch.cuh.  For the time of a launch the lattice is kept as an
+// of escg_patch.cuh.  For the time of a call the lattice is kept as an
 // array of macros, row slot ky, column slot kx at ky * GQ + kx (a byte or two
 // bytes for 2 x 2 sites): macro_fill_kernel makes it from the caller's array
-// before the launch and macro_drain_kernel writes the caller's array after
-// it.  A block's tile is the 33 x 33 macros of its joint slots -- 1.1 or 2.2 KB,
+// before the call's first launch and macro_drain_kernel writes the caller's
+// array after its last.  A block's tile is the 33 x 33 macros of its joint slots -- 1.1 or 2.2 KB,
 // one 16-byte load per thread, no conversion -- and holds its 64 x 64 sites,
 // its rim lines and its corners, so the Moore rule needs nothing more.  At
 // L = 12800 the macros are 41 or 82 MB and stay in the L2, where the array of
@@ -754,19 +754,20 @@ cudaError_t launch_persistent_macro(const PersistentArgs& args, int grid, cudaSt
   a.rcp_per = div_rcp32(nb >> 2);
   a.rcp_half = div_rcp32((uint32_t)(a.d.P >> 1));
   const bool any = !a.d.blocks64;
-  cudaError_t e = any ? launch_macro_fill_any(a.d, a.macros, a.st, stream)
-                      : launch_macro_fill(a.d, a.macros, a.st, stream);
+  cudaError_t e = cudaSuccess;
+  if (a.fill)
+    e = any ? launch_macro_fill_any(a.d, a.macros, a.st, stream) : launch_macro_fill(a.d, a.macros, a.st, stream);
   if (e != cudaSuccess) return e;
   if (any) {
     int nsx = axis_slots(a.d.ax, a.d.P), nsy = axis_slots(a.d.ay, a.d.Py), gp = macro_pitch(a.d);
     void* params[] = {&a, &nsx, &nsy, &gp};
     e = cudaLaunchKernel(macro_any_fn(a.d), dim3(grid), dim3(256), params, 0, stream);
-    return e != cudaSuccess ? e : launch_macro_drain_any(a.d, a.macros, a.st, stream);
+  } else {
+    void* params[] = {&a};
+    e = cudaLaunchKernel(macro_kernel_fn(a.d, a.threads), dim3(grid), dim3(a.threads), params, 0, stream);
   }
-  void* params[] = {&a};
-  e = cudaLaunchKernel(macro_kernel_fn(a.d, a.threads), dim3(grid), dim3(a.threads), params, 0, stream);
-  if (e != cudaSuccess) return e;
-  return launch_macro_drain(a.d, a.macros, a.st, stream);
+  if (e != cudaSuccess || !a.drain) return e;
+  return any ? launch_macro_drain_any(a.d, a.macros, a.st, stream) : launch_macro_drain(a.d, a.macros, a.st, stream);
 }
 
 }  // namespace escg_impl

@@ -763,13 +763,15 @@ cudaError_t launch_persistent_group(const PersistentArgs& a, const GroupConfig& 
   arg.gqy = fine_rows(a.d);
   arg.nsx = axis_slots(a.d.ax, a.d.P);
   arg.nsy = axis_slots(a.d.ay, a.d.Py);
-  cudaError_t e = a.d.blocks64 ? launch_macro_fill(a.d, a.macros, a.st, stream)
-                                  : launch_macro_fill_any(a.d, a.macros, a.st, stream);
+  cudaError_t e = cudaSuccess;
+  if (a.fill)
+    e = a.d.blocks64 ? launch_macro_fill(a.d, a.macros, a.st, stream)
+                     : launch_macro_fill_any(a.d, a.macros, a.st, stream);
   if (e != cudaSuccess) return e;
   void* params[] = {&arg};
   e = cudaLaunchCooperativeKernel(group_fn(a.d, cfg.groups), dim3((a.d.P / 2) * (a.d.Py / 2)), dim3(cfg.groups * cfg.group_threads),
                                   params, (size_t)cfg.dyn_bytes, stream);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || !a.drain) return e;
   return a.d.blocks64 ? launch_macro_drain(a.d, a.macros, a.st, stream)
                       : launch_macro_drain_any(a.d, a.macros, a.st, stream);
 }

@@ -90,6 +90,7 @@ struct PersistentArgs {
   int32_t threads;         // flag kernel on macros: 128 (two sub-blocks per thread, up to 8
                            // CTAs per SM) or 256 (one)
   void* macros;            // macro array (escg_flag.cu, escg_group.cu)
+  int32_t fill, drain;     // whether the launch starts with the lattice array and ends with it
   // div_rcp32 of the ticket decode's divisors (blocks per MCS, blocks per
   // coarse phase, half the blocks per row); filled in by launch_persistent
   uint32_t rcp_nb, rcp_per, rcp_half;
@@ -108,9 +109,9 @@ cudaError_t launch_macro_fill(const LatticeDesc& d, void* macros, RunState* st, 
 cudaError_t launch_macro_drain(const LatticeDesc& d, const void* macros, const RunState* st, cudaStream_t stream);
 cudaError_t launch_macro_fill_any(const LatticeDesc& d, void* macros, RunState* st, cudaStream_t stream);
 cudaError_t launch_macro_drain_any(const LatticeDesc& d, const void* macros, const RunState* st, cudaStream_t stream);
-// The flag kernel on macros (uniform partitions, any rule; escg_flag.cu): the
-// lattice array is turned into a.macros, run there by CTAs of a.threads and
-// written back.  Grid by occupancy.
+// The flag kernel on macros (uniform partitions, any rule; escg_flag.cu): with
+// a.fill the lattice array is turned into a.macros, CTAs of a.threads run
+// there, with a.drain it is written back.  Grid by occupancy.
 int persistent_macro_grid(const LatticeDesc& d, int device, int threads);
 // The same for other partitions (256 threads): 0 where it cannot run.
 int persistent_macro_any_grid(const LatticeDesc& d, int device);

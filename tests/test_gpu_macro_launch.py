@@ -41,3 +41,42 @@ def test_a_refused_lattice_stays_as_it_was_given(L, S, kw):
     o, _ = O.replay_run(lat, D, 1.0, 1.0, 2.0, 4, 3, neighbourhood=kw.get("neighbourhood", 4))
     assert np.array_equal(g.snapshot(), o)
     g.close()
+
+
+@pytest.mark.parametrize("L,S,kw", CASES)
+@pytest.mark.parametrize("stop", [False, True])
+def test_a_call_of_many_launches_converts_once(L, S, kw, stop):
+    """A run that stops at extinction has a launch for every log point: one
+    conversion each way for the call, its lattice and its log as the oracle's."""
+    D, g = _lattice(L, S, 8, log_every=1, stop_at_extinction=stop, **kw)
+    rule = dict(neighbourhood=kw.get("neighbourhood", 4))
+    lat = O.init(L, S, 0.2, 8)
+    before = g.launches
+    g.run(11)
+    assert g.launches - before == (13 if stop else 3)
+    o, _ = O.replay_run(lat, D, 1.0, 1.0, 2.0, 8, 11, **rule)
+    assert np.array_equal(g.snapshot(), o)
+    _, log = g.counts_log()
+    _, olog, _ = O.run_observed(lat, D, 1.0, 1.0, 2.0, 8, 11, log_every=1, **rule)
+    assert np.array_equal(log, olog)
+    g.close()
+
+
+@pytest.mark.parametrize("L,kw", [(128, dict(persistent=3)), (201, {}), (200, dict(neighbourhood=8)),
+                                  (400, dict(persistent=3)), (384, dict(neighbourhood=8))])
+def test_extinction_within_a_call(L, kw):
+    """The call stops where the oracle stops, and the array holds that lattice."""
+    D = O.circulant(3, (1,))   # a few sites of 2 among 1, which beats it
+    rule = dict(neighbourhood=kw.get("neighbourhood", 4))
+    lat = np.ones((L, L), dtype=np.uint8)
+    lat[3::L // 5, 5::L // 4] = 2
+    g = E.Lattice(L, 3, D, (1.0, 1.0, 1.0), 3, log_every=1, stop_at_extinction=True, **kw)
+    g.restore(lat, 0)
+    o, log, mend = O.run_observed(lat, D, 1.0, 1.0, 1.0, 3, 400, log_every=1, stop_at_extinction=True, **rule)
+    assert 1 < mend < 400
+    g.run(400)
+    assert g.mcs == mend
+    assert np.array_equal(g.snapshot(), o)
+    g.run(5)   # stopped: nothing moves
+    assert g.mcs == mend and np.array_equal(g.snapshot(), o)
+    g.close()
