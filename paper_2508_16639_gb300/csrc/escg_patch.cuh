@@ -161,17 +161,39 @@ __device__ __forceinline__ void patch_tables_fill(PatchTables& T, const LatticeD
 // Mirrors entry e of a w-wide, h-high sub-block whose sides `edge` (1 top,
 // 2 bottom, 4 left, 8 right) are edges of a reflecting lattice: a step that
 // would leave the lattice goes the other way in that coordinate.
-__device__ __forceinline__ uint32_t patch_mirror(uint32_t e, int w, int h, int lg, uint32_t edge) {
+__host__ __device__ constexpr uint32_t patch_mirror(uint32_t e, int w, int h, int lg, uint32_t edge) {
   const uint32_t dir = e & ((1u << lg) - 1u), site = e >> lg;
   const int r = (int)(site / (uint32_t)w), c = (int)site - r * w;
-  int dr, dc;
-  dir_step(dir, &dr, &dc);
+  int dr = (int)((0xA058u >> (2 * dir)) & 3u) - 1, dc = (int)((0x8885u >> (2 * dir)) & 3u) - 1;   // dir_step
   if (((edge & 1u) && r == 0 && dr < 0) || ((edge & 2u) && r == h - 1 && dr > 0)) dr = -dr;
   if (((edge & 4u) && c == 0 && dc < 0) || ((edge & 8u) && c == w - 1 && dc > 0)) dc = -dc;
   // directions by 3 (dr + 1) + dc + 1: 4 0 5 2 . 3 6 1 7
   const uint32_t nd = (uint32_t)(0x716302504ull >> (4 * (3 * (dr + 1) + dc + 1))) & 15u;
   return (site << lg) | nd;
 }
+
+// The same for every entry and edge, by neighbourhood: 2 x 2 from entry 0, then
+// the shapes of PatchTables::irr.  A mirrored step is one load here (6 KB, in
+// the L1 of every SM that runs such a lattice); worked out step by step, with a
+// division by w, it took longer than the step itself.  us per MCS of reflecting
+// lattices, byte kernels, worked out, table: L = 100 34.6, 31.0, 12.3; 150 (S = 5)
+// 39.5, 49.2, 33.0; 191 39.5, 41.4, 29.7; 3200 26.9, 25.3, 23.0, (S = 5) 27.1, 28.2,
+// 26.2.
+struct MirrorTable {
+  uint8_t e[2][16][25 * kPatchMaxNbh];
+};
+constexpr MirrorTable make_mirror_table() {
+  MirrorTable t{};
+  constexpr int kShape[4][3] = {{0, 2, 2}, {4, 3, 2}, {10, 2, 3}, {16, 3, 3}};   // first site, width, height
+  for (int lg = 2; lg <= 3; ++lg)
+    for (uint32_t edge = 0; edge < 16u; ++edge)
+      for (int k = 0; k < 4; ++k)
+        for (int e = 0; e < (kShape[k][1] * kShape[k][2]) << lg; ++e)
+          t.e[lg - 2][edge][(kShape[k][0] << lg) + e] =
+              (uint8_t)patch_mirror((uint32_t)e, kShape[k][1], kShape[k][2], lg, edge);
+  return t;
+}
+static __device__ const MirrorTable g_mirror = make_mirror_table();
 
 // The four attempts of a 2 x 2 sub-block as the tables give them from the
 // random words alone: L the pair's entry (swap if `general` is false, else
@@ -196,7 +218,7 @@ __device__ __forceinline__ Steps2<PL> patch_steps2(uint4 x, const PatchTables& T
 #pragma unroll
   for (int t = 0; t < 4; ++t) {
     e[t] = w[t] >> (30 - LG);
-    if (REFLECT && edge) e[t] = patch_mirror(e[t], 2, 2, LG, edge);
+    if (REFLECT && edge) e[t] = g_mirror.e[LG - 2][edge][e[t]];
     u[t] = w[t] << (2 + LG);
   }
   // one choice for the lanes that come here together: a mixed warp would
@@ -262,15 +284,12 @@ __device__ __forceinline__ void patch_run2(uint32_t (&v)[PL], const Steps2<PL>& 
   }
 }
 
-// One attempt (word w) of a sub-block with a 3-site side; n = nbh w h, lut
-// the shape's entries.  V, W: its bits (PL = 1: V alone).
-template <int PL, int LG, bool REFLECT>
-__device__ __forceinline__ void patch_attempt(uint64_t& V, uint64_t& W, uint32_t w, uint32_t n,
+// One attempt (entry e, action draw u) of a sub-block with a 3-site side; lut the
+// shape's entries.  V, W: its bits (PL = 1: V alone).
+template <int PL>
+__device__ __forceinline__ void patch_attempt(uint64_t& V, uint64_t& W, uint32_t e, uint32_t u,
                                               const uint2* __restrict__ lut, const PatchTables& T, uint32_t tx,
-                                              uint32_t txi, int pw, int ph, uint32_t edge) {
-  uint32_t e = __umulhi(w, n);
-  const uint32_t u = w * n;
-  if (REFLECT && edge) e = patch_mirror(e, pw, ph, LG, edge);
+                                              uint32_t txi) {
   const uint2 L = lut[e];
   const uint32_t act = u < tx ? 0u : (u < txi ? 1u : 2u);
   if (PL == 1) {
@@ -333,12 +352,25 @@ __device__ __forceinline__ void patch_store2(typename MacroOf<PL>::type* __restr
   }
 }
 
+// Entries of a sub-block with a 3-site side: nbh times its sites, and the first
+// of its shape in PatchTables::irr.
+template <int LG>
+__device__ __forceinline__ uint32_t patch_entries(bool wc, bool wr) {
+  return (uint32_t)((wc ? 3 : 2) * (wr ? 3 : 2)) << LG;
+}
+template <int LG>
+__device__ __forceinline__ uint32_t patch_first(bool wc, bool wr) {
+  return !wr ? 0u : (!wc ? 6u << LG : 12u << LG);
+}
+
 // All attempts (words w[0 .. 5] or w[0 .. 8]) of a sub-block with a 3-site
-// side (wc: 3 wide, wr: 3 high), from and to its macros.
+// side (wc: 3 wide, wr: 3 high), from and to its macros.  REFLECT: their entries
+// are the bytes of ent, else the words give them.
 template <int PL, int LG, bool REFLECT>
 __device__ __forceinline__ void patch_irregular(typename MacroOf<PL>::type* __restrict__ M, int i00, int dc, int dr,
                                                 int pitch, bool wc, bool wr, const uint32_t (&w)[9],
-                                                const PatchTables& T, uint32_t tx, uint32_t txi, uint32_t edge) {
+                                                const uint32_t (&ent)[3], const PatchTables& T, uint32_t tx,
+                                                uint32_t txi) {
   typedef typename MacroOf<PL>::type MT;
   constexpr int kB = 8 * PL;                          // bits of a macro
   constexpr uint32_t kMid = PL == 1 ? 0x33u : 0x0F0Fu;   // sites of a middle column's macro
@@ -361,13 +393,13 @@ __device__ __forceinline__ void patch_irregular(typename MacroOf<PL>::type* __re
     V = ((uint64_t)lo[PL - 1] << 32) | lo[0];
     W = ((uint64_t)(m2 | (m3 << 16)) << 32) | (m0 | (m1 << 16));
   }
-  const int pw = wc ? 3 : 2, ph = wr ? 3 : 2;
-  const uint32_t n = (uint32_t)(pw * ph) << LG;
-  const uint2* lut = T.irr + (ph == 2 ? 0 : (pw == 2 ? 6 << LG : 12 << LG));
+  const uint32_t n = patch_entries<LG>(wc, wr);
+  const uint2* lut = T.irr + patch_first<LG>(wc, wr);
 #pragma unroll
   for (int t = 0; t < 9; ++t) {
     if (t >= 6 && !(wc && wr)) break;
-    patch_attempt<PL, LG, REFLECT>(V, W, w[t], n, lut, T, tx, txi, pw, ph, edge);
+    const uint32_t e = REFLECT ? (ent[t >> 2] >> (8 * (t & 3))) & 255u : __umulhi(w[t], n);
+    patch_attempt<PL>(V, W, e, w[t] * n, lut, T, tx, txi);
   }
   lo[0] = (uint32_t)V;
   if (PL == 2) lo[PL - 1] = (uint32_t)(V >> 32);
@@ -426,7 +458,8 @@ __host__ __device__ __forceinline__ uint4 philox_step(const StepKeys& k, uint32_
 
 // One sub-block of a fine phase with what is known of it before the phase:
 // for a 2 x 2 one its steps, for one with a 3-site side its random words, in
-// the same registers (word t in s.L[t / 2], the last one in i8).
+// the same registers (word t in s.L[t / 2], the last one in i8; with a
+// reflecting boundary the entries in s.A).
 template <int PL>
 struct PatchItem {
   Steps2<PL> s;
@@ -460,6 +493,22 @@ __device__ __forceinline__ void patch_item_draw(PatchItem<PL>& I, const StepKeys
     I.s.L[2] = make_uint2(y.x, y.y);
     I.s.L[3] = make_uint2(y.z, y.w);
     I.i8 = z.x;
+    if (REFLECT) {
+      // the entries now: a mirrored one must not wait in the chain of the steps
+      const bool wc = (I.fl & 2u) != 0u, wr = (I.fl & 4u) != 0u;
+      const uint32_t n = patch_entries<LG>(wc, wr), edge = I.fl >> 4;
+      const uint32_t w[9] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, z.x};
+      const uint8_t* mir = g_mirror.e[LG - 2][edge] + (4u << LG) + patch_first<LG>(wc, wr);
+      uint32_t ent[3] = {0u, 0u, 0u};
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        uint32_t e = __umulhi(w[t], n);
+        if (edge) e = mir[e];
+        ent[t >> 2] |= e << (8 * (t & 3));
+      }
+      I.s.A[0] = make_uint2(ent[0], ent[1]);
+      I.s.A[1].x = ent[2];
+    }
   }
 }
 
@@ -476,8 +525,9 @@ __device__ __forceinline__ void patch_item_run(typename MacroOf<PL>::type* __res
   } else {
     const uint32_t w[9] = {I.s.L[0].x, I.s.L[0].y, I.s.L[1].x, I.s.L[1].y, I.s.L[2].x, I.s.L[2].y, I.s.L[3].x,
                            I.s.L[3].y, I.i8};
-    patch_irregular<PL, LG, REFLECT>(M, I.i00, I.dc, I.dr, pitch, (I.fl & 2u) != 0u, (I.fl & 4u) != 0u, w, T, tx, txi,
-                                     REFLECT ? I.fl >> 4 : 0u);
+    const uint32_t ent[3] = {I.s.A[0].x, I.s.A[0].y, I.s.A[1].x};
+    patch_irregular<PL, LG, REFLECT>(M, I.i00, I.dc, I.dr, pitch, (I.fl & 2u) != 0u, (I.fl & 4u) != 0u, w, ent, T, tx,
+                                     txi);
   }
 }
 
