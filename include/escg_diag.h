@@ -75,6 +75,14 @@ int32_t escg_coarse_blocks(escg_t* h);
  * for a NULL handle.  The choice never changes results. */
 const char* escg_update_kernel(escg_t* h);
 
+/* What the kernels of a call escg_run(h, n_mcs) step: "bytes", the lattice array
+ * (one byte per site, also where the array is packed), or "macros", its sites
+ * in the 2 x 2 groups of the kernels on macros, which have the names of the ones
+ * on bytes.  Short calls stay on bytes, for they would pay more for the two
+ * conversions than they win.  A static string, "" for a NULL handle; results
+ * never depend on it. */
+const char* escg_run_layout(escg_t* h, uint64_t n_mcs);
+
 #ifdef __cplusplus
 }
 #endif

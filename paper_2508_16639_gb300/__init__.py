@@ -248,6 +248,10 @@ class Lattice:
         """Name of the kernel that advances this lattice (fixed at creation)."""
         return load().escg_update_kernel(self._h).decode()
 
+    def run_layout(self, n_mcs: int) -> str:
+        """What run(n_mcs) steps: "bytes" (the lattice array) or "macros"."""
+        return load().escg_run_layout(self._h, int(n_mcs)).decode()
+
     @property
     def mcs(self) -> int:
         return int(load().escg_current_mcs(self._h))

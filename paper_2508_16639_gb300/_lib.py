@@ -115,6 +115,7 @@ SIGNATURES = {
     "escg_debug_graph_builds": (C.c_int32, [C.c_void_p]),
     "escg_coarse_blocks": (C.c_int32, [C.c_void_p]),
     "escg_update_kernel": (C.c_char_p, [C.c_void_p]),
+    "escg_run_layout": (C.c_char_p, [C.c_void_p, C.c_uint64]),
     "escg_diag_alg_throughput": (C.c_int, [C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     "escg_autotune_result": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                        C.POINTER(C.c_double), C.POINTER(C.c_int32)]),

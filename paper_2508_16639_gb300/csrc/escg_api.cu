@@ -3,6 +3,7 @@
 // table, the initial lattice) and run orchestration on the handle's stream.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -260,8 +261,14 @@ struct escg {
   int own_dyn = 0;               // its shared-memory padding
   int own_threads = 0;           // and CTA size
   int flag_threads = 256;        // CTA size of the flag kernel (128: uniform geometry, > 4 CTAs per SM)
-  bool use_macro = false;        // flag kernel on macros (uniform geometry)
+  bool use_macro = false;        // flag kernel on macros
   void* d_macros = nullptr;      // its macro array, kept for the handle's life
+  // Calls of fewer than macro_min MCS on a handle with use_macro or use_group:
+  // the byte owners (gown), else the flag kernel on bytes.
+  uint32_t macro_min = 1;
+  bool brief_gown = false;
+  int brief_grid = 0, brief_threads = 256;
+  uint64_t done_mcs = 0;         // MCS that the block epochs d_done stand at (the owners leave them)
   bool use_gown = false;         // block owners on a generic partition
   int tuned_mode = 0, tuned_ctas = 0;   // autotuner's choice (launch mode, CTAs per SM)
   double tuned_ms_per_mcs = 0.0;
@@ -388,6 +395,7 @@ int reset_state(escg* h, uint64_t mcs, bool validate = false) {
   // for (a lattice restored at an MCS the handle has run through before):
   // epoch 0 never matches a wait, which always expects an epoch >= 1.
   if (h->d_ob) CUDA_TRY(cudaMemsetAsync(h->d_ob, 0, h->ob_words * sizeof(unsigned long long), h->stream));
+  h->done_mcs = mcs;
   h->log_num0_host = num0;
   h->mcs_enq = mcs;
   h->failed = false;
@@ -473,8 +481,8 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   h->own_dyn = h->own_threads = 0;
   h->gown = GownConfig{};
   h->group = GroupConfig{};
-  h->use_macro = false;
-  h->grid = persistent_grid(h->device, d.uniform64 != 0 && h->bits == 8);
+  h->use_macro = h->brief_gown = false;
+  h->grid = persistent_grid(h->device, d.uniform64 != 0 || flag_variant(d));
   // the TMA and mailbox kernels are written for square lattices of one byte
   // per site; the flag kernel takes rectangular and packed ones in both
   // geometries
@@ -542,6 +550,7 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
     if (persistent_group_config(d, h->device, &cfg, ctas_per_sm) > 0 &&
         (persistent == 5 || cfg.ctas_per_sm <= kGownDefaultPerSM) && ensure_macros(h)) {
       if (ensure_records(h, (size_t)p.P * py.P * kGroupRecordWords) != ESCG_OK) return ESCG_ENOMEM;
+      h->brief_gown = h->use_gown;
       h->use_group = h->use_gown = true;
       h->group = cfg;
     }
@@ -556,33 +565,50 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
     h->use_resident = true;
     h->use_own = h->use_gown = h->use_group = false;
   }
-  // The flag kernel on a uniform lattice (any bits per site) with more than
-  // 4 CTAs per SM requested, or by default (1) with at least kFlag128Ratio times as many
-  // blocks per coarse phase as 256-thread CTAs: the 128-thread build (two
-  // quads per thread), up to 8 per SM.  Measured (µs per MCS, 4 x 256 vs
-  // 8 x 128 threads per SM): L = 2048 21.7 vs 26.7, 3200 25.5 vs 32.8 (5 x 128:
+  // The flag kernel on bytes on a uniform lattice (any bits per site) with more
+  // than 4 CTAs per SM requested, or by default (1) with at least kFlag128Ratio
+  // times as many blocks per coarse phase as 256-thread CTAs: the 128-thread
+  // build (two quads per thread), up to 8 per SM.  Measured (µs per MCS, 4 x 256
+  // vs 8 x 128 threads per SM): L = 2048 21.7 vs 26.7, 3200 25.5 vs 32.8 (5 x 128:
   // 28.9), 6400 91.4 vs 78.7 -- more visits in flight pay once the phases are
-  // several waves deep and throughput, not the colour chain, binds.
+  // several waves deep and throughput, not the colour chain, binds.  The same
+  // rule holds on macros.
   h->flag_threads = 256;
   const bool flag = !h->use_tma && !h->use_ll && !h->use_own && !h->use_gown && !h->use_resident;
-  if (flag && persistent != 0 && d.blocks64 && ensure_macros(h)) {
-    h->use_macro = true;
-    h->grid = persistent_macro_grid(d, h->device, 256);
-    const bool deep = persistent == 1 && (int64_t)p.P * py.P / 4 >= (int64_t)kFlag128Ratio * h->grid;
-    if (ctas_per_sm > 4 || deep) {
-      h->flag_threads = 128;
-      h->grid = persistent_macro_grid(d, h->device, 128);
+  auto wide_ctas = [&](int grid) {
+    return ctas_per_sm > 4 || (persistent == 1 && (int64_t)p.P * py.P / 4 >= (int64_t)kFlag128Ratio * grid);
+  };
+  const bool bytes = flag || h->use_group;   // the flag kernel on bytes, for all or for short calls
+  if (bytes && d.uniform64 && wide_ctas(h->grid)) {
+    h->flag_threads = 128;
+    h->grid = persistent_grid128(h->device);
+  }
+  h->brief_grid = h->grid;
+  h->brief_threads = h->flag_threads;
+  // The flag kernel on macros, uniform partitions and others
+  if (flag && persistent != 0) {
+    int grid = 0, threads = 256;
+    if (d.blocks64) {
+      grid = persistent_macro_grid(d, h->device, 256);
+      if (wide_ctas(grid)) {
+        threads = 128;
+        grid = persistent_macro_grid(d, h->device, 128);
+      }
+    } else {
+      grid = persistent_macro_any_grid(d, h->device);
+    }
+    if (grid > 0 && ensure_macros(h)) {
+      h->use_macro = true;
+      h->grid = grid;
+      h->flag_threads = threads;
     }
   }
-  // The flag kernel on macros, any other partition
-  if (flag && persistent != 0 && !d.blocks64 && persistent_macro_any_grid(d, h->device) > 0 && ensure_macros(h)) {
-    h->use_macro = true;
-    h->grid = persistent_macro_any_grid(d, h->device);
-  }
+  h->macro_min = h->use_macro || h->use_group ? macro_min_mcs(d, h->use_group, h->flag_threads == 128) : 1;
   if (ctas_per_sm > 0) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (sms * ctas_per_sm < h->grid) h->grid = sms * ctas_per_sm;
+    h->grid = std::min(h->grid, sms * ctas_per_sm);
+    h->brief_grid = std::min(h->brief_grid, sms * ctas_per_sm);
   }
 
   return ESCG_OK;
@@ -906,9 +932,16 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
     return ESCG_EINVAL;
   }
   const uint32_t k = h->opt.log_every;
+  // a call too short for the conversions stays on the lattice array
+  const bool brief = (h->use_macro || h->use_group) && n_mcs < h->macro_min;
+  const bool macro = h->use_macro && !brief, group = h->use_group && !brief;
+  const bool gown = brief ? h->brief_gown : h->use_gown;
   // rule variants count log points with the count kernel between launches
-  // (the resident kernel and the one on macros count in-kernel for every rule)
-  const bool fused = (h->desc.nbh == 4 && !h->desc.reflect) || h->use_resident || h->use_macro || h->use_group;
+  // (the resident kernel and the ones on macros count in-kernel for every rule)
+  const bool fused = (h->desc.nbh == 4 && !h->desc.reflect) || h->use_resident || macro || group;
+  // the kernels that keep the block epochs: all but the owners and the resident
+  // ones, whose launches leave them behind
+  const bool epochs = !h->use_resident && !group && !h->use_own && !gown && h->opt.persistent;
   // Nothing reads the lattice array between the launches of a call on macros:
   // it is turned into macros before the first and written after the last.
   // Runs to extinction that log every MCS, a launch each, us per MCS with the
@@ -928,12 +961,13 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
     }
     // the persistent kernel numbers work items with 32-bit tickets
     const uint64_t per_mcs = (uint64_t)h->part.P * h->part_y.P;
-    const uint64_t max_chunk = ((1ull << 31) - (uint64_t)h->grid) / per_mcs;
+    const int max_grid = brief ? h->brief_grid : h->grid;
+    const uint64_t max_chunk = ((1ull << 31) - (uint64_t)max_grid) / per_mcs;
     if (end - h->mcs_enq > max_chunk) end = h->mcs_enq + max_chunk;
     const uint32_t m0 = (uint32_t)h->mcs_enq, n = (uint32_t)(end - h->mcs_enq);
     if (h->opt.persistent) {
       const uint64_t items = (uint64_t)n * per_mcs;
-      const int grid = (int)(items < (uint64_t)h->grid ? items : (uint64_t)h->grid);
+      const int grid = (int)(items < (uint64_t)max_grid ? items : (uint64_t)max_grid);
       PersistentArgs a{};
       a.d = h->desc;
       a.st = h->d_state;
@@ -947,19 +981,23 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
       a.stall_block = h->stall_block;
       a.ob = h->d_ob;
       a.fuse_counts = fused ? 1 : 0;
-      a.threads = h->flag_threads;
+      a.threads = brief ? h->brief_threads : h->flag_threads;
       a.macros = h->d_macros;
       a.fill = m0 == start ? 1 : 0;
       a.drain = end == target ? 1 : 0;
+      if (epochs && h->done_mcs != m0) {
+        CUDA_TRY(launch_fill_u32(h->d_done, h->part.P * h->part_y.P, m0, h->stream));
+        h->launches++;
+      }
       CUDA_TRY(timing_begin(h));
       if (h->use_resident) {
         CUDA_TRY(launch_resident(a, h->stream));
-      } else if (h->use_group) {
+      } else if (group) {
         CUDA_TRY(launch_persistent_group(a, h->group, h->stream));
         h->launches += a.fill + a.drain;
       } else if (h->use_own) {
         CUDA_TRY(launch_persistent_own(a, h->own_dyn, h->own_threads, h->stream));
-      } else if (h->use_gown) {
+      } else if (gown) {
         CUDA_TRY(launch_persistent_gown(a, h->gown, h->stream));
       } else if (h->use_tma) {
         TmaArgs ta{};
@@ -968,7 +1006,7 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
         CUDA_TRY(launch_persistent_tma(ta, grid, h->stream));
       } else if (h->use_ll) {
         CUDA_TRY(launch_persistent_ll(a, grid, h->stream));
-      } else if (h->use_macro) {
+      } else if (macro) {
         CUDA_TRY(launch_persistent_macro(a, grid, h->stream));
         h->launches += a.fill + a.drain;
       } else {
@@ -976,6 +1014,7 @@ int escg_run(escg_t* h, uint64_t n_mcs) {
       }
       CUDA_TRY(timing_end(h));
       h->launches++;
+      if (epochs) h->done_mcs = end;
       if (h->use_ll) {
         CUDA_TRY(launch_ll_merge(h->desc, h->d_ob, h->d_state, (uint32_t)end, h->stream));
         h->launches++;
@@ -1250,6 +1289,12 @@ const char* escg_update_kernel(escg_t* h) {
   if (h->use_gown) return "persistent_gown_kernel";
   if (h->use_tma) return "persistent_tma_kernel";
   return h->use_ll ? "persistent_ll_kernel" : "persistent_kernel";
+}
+
+const char* escg_run_layout(escg_t* h, uint64_t n_mcs) {
+  if (!h) return "";
+  const bool macros = h->use_resident ? resident_on_macros(h->desc) : (h->use_macro || h->use_group) && n_mcs >= h->macro_min;
+  return macros ? "macros" : "bytes";
 }
 
 void escg_destroy(escg_t* h) { free_handle(h); }

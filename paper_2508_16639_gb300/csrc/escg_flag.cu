@@ -747,6 +747,38 @@ int persistent_macro_grid(const LatticeDesc& d, int device, int threads) {
   return sms * (occ < cap ? occ : cap);
 }
 
+// A call pays for two conversions (15 us at L = 3200, 300 at 12700), which the
+// macros win back at some us per MCS.  Calls below the lines run on bytes.  us per
+// MCS of calls of n MCS on bytes and on macros (M = 1e-4 unless stated), the line
+// where they meet:
+//  * owners: L = 800 n = 1 40.4, 47.5, n = 2 31.7, 32.4, n = 5 26.8, 23.5; L = 2200 Moore
+//    53.5, 64.9 / 45.0, 45.7 / 40.5, 33.8.  On 64 x 64 blocks with a reflecting
+//    boundary n = 1 already gains (L = 1024 1.15 x).
+//  * flags, 64 x 64 blocks, 2 bits per site: L = 3200 34.1, 39.6 / 29.4, 29.1 / 25.3,
+//    22.7; the Moore bytes are slower and meet at 1 (39.3, 40.5), deep phases (L = 6400)
+//    too.
+//  * the same at 4 bits: L = 3200 meets at 5 to 8 (26.5 each at n = 5), Moore at 3,
+//    reflecting at 5; deep ones at 2 (82.8, 81.2).  With few exchanges (M = 0: every
+//    step takes the rule table) the macros gain 0 to 5 % at n = 20 and lose at 10.
+//  * packed lattices: the bytes pay a conversion in every visit; the rule variants
+//    and ragged blocks always gain (L = 3333, 2 bits, n = 1 1.3 x).
+//  * other partitions: L = 3333 56.4, 72.6 / 51.6, 52.7 / n = 3 1.08 x; L = 12700 629, 689 /
+//    624, 540.
+uint32_t macro_min_mcs(const LatticeDesc& d, bool group, bool deep) {
+  const bool one = patch_planes(d) == 1, moore = d.nbh == 8, refl = d.reflect != 0;
+  if (group) return d.blocks64 && refl ? 1u : 2u;
+  if (!d.blocks64) return d.bits != 8 ? 1u : ((size_t)d.H * d.L >= (32u << 20) ? 2u : 3u);
+  const bool few = d.tx < 0x80000000u;   // fewer than half the attempts exchange
+  if (d.bits != 8) {
+    if (moore || refl) return 1u;
+    return one ? (deep ? 1u : 2u) : (few ? 5u : (deep ? 2u : 3u));
+  }
+  if (one) return deep || (moore && !refl) ? 1u : 2u;
+  if (refl) return moore && deep ? 3u : 5u;
+  if (moore) return deep ? 1u : 3u;
+  return few ? 16u : (deep ? 2u : 6u);
+}
+
 cudaError_t launch_persistent_macro(const PersistentArgs& args, int grid, cudaStream_t stream) {
   PersistentArgs a = args;
   const uint32_t nb = (uint32_t)(a.d.P * a.d.Py);

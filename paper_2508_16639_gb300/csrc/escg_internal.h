@@ -87,8 +87,8 @@ struct PersistentArgs {
   int32_t stall_block;   // test hook: never publish this block's epoch (-1: off)
   unsigned long long* ob;  // boundary records of the mailbox kernel ([P*P][4][32]), else null
   int32_t fuse_counts;     // 1: counts of log points fused into the visits; 0: the host counts
-  int32_t threads;         // flag kernel on macros: 128 (two sub-blocks per thread, up to 8
-                           // CTAs per SM) or 256 (one)
+  int32_t threads;         // flag kernel on uniform partitions: 128 (two quads per thread, up to
+                           // 8 CTAs per SM) or 0 / 256 (one)
   void* macros;            // macro array (escg_flag.cu, escg_group.cu)
   int32_t fill, drain;     // whether the launch starts with the lattice array and ends with it
   // div_rcp32 of the ticket decode's divisors (blocks per MCS, blocks per
@@ -100,6 +100,15 @@ struct PersistentArgs {
 cudaError_t launch_persistent(const PersistentArgs& a, int grid, cudaStream_t stream);
 // Occupancy-derived grid size of the persistent kernel for a lattice.
 int persistent_grid(int device, bool uniform);
+// The same for the 128-thread build of the uniform flag kernel (up to 8 per SM).
+int persistent_grid128(int device);
+// A rule variant that the flag kernel on bytes has uniform builds for.
+inline bool flag_variant(const LatticeDesc& d) {
+  return d.blocks64 && d.bits == 8 && (d.nbh == 8 || d.reflect);
+}
+// The shortest call (in MCS) that runs on macros; `group`: the owners, `deep`:
+// the 128-thread CTAs of the flag kernel.
+uint32_t macro_min_mcs(const LatticeDesc& d, bool group, bool deep);
 // The macro array of a lattice (escg_patch.cuh): rows of macro_pitch macros.
 // Lattice array <-> macros, for uniform partitions and for any.  A stopped
 // lattice is left alone: it may hold values that no macro does.
@@ -120,6 +129,8 @@ cudaError_t launch_persistent_macro(const PersistentArgs& a, int grid, cudaStrea
 // Whole-lattice residency: one CTA runs MCS [m_begin, m_begin + n_mcs) with
 // the lattice in shared memory (counts of log points written in-kernel).
 bool resident_fits(const LatticeDesc& d, int device);
+// Whether it does so on macros (escg_resident_patch.cuh) or on the byte image.
+bool resident_on_macros(const LatticeDesc& d);
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream);
 
 // Uniform geometry, boundary-mailbox variant (the default persistent path):

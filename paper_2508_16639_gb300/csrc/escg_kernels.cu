@@ -200,26 +200,34 @@ constexpr int kUniLaunchPerSM = 4;
 __device__ __forceinline__ void own_fine_phases(const LatticeDesc& d, int bx, int by, uint32_t m, uint8_t* tile,
                                                 uint32_t ord, const uint8_t* trans);
 
-// One quad (2 x 2 sub-blocks) per thread, up to 4 CTAs per SM.  Handles on
-// uniform partitions run the same flags on macros (escg_flag.cu); the UNI
-// build here serves callers that leave no memory for them.
-template <bool UNI, bool PACKED>
-__global__ void __launch_bounds__(kPersistentThreads, UNI ? kUniMinBlocks : 4) persistent_kernel(PersistentArgs a) {
-  static_assert(!(UNI && PACKED), "packed lattices: the generic visit");
-  constexpr int NT = kPersistentThreads;
+// NT = 256: one quad (2 x 2 sub-blocks) per thread, up to 4 CTAs per SM;
+// NT = 128 (uniform geometry, any bits per site): two quads per thread
+// stepped pairwise (own_fine_phases), up to 8 CTAs per SM -- twice the
+// visits in flight per SM for the same number of threads.
+// VAR (uniform geometry, one byte per site): a rule variant on 64 x 64
+// blocks -- bit 0 a reflecting boundary, bit 1 the Moore neighbourhood.
+// Long calls run the same flags on macros (escg_flag.cu); these builds take the
+// calls that are too short for its conversions (macro_min_mcs) and the lattices
+// that leave no memory for macros.
+template <bool UNI, bool PACKED = false, int NT = kPersistentThreads, int VAR = 0>
+__global__ void __launch_bounds__(NT, NT == 128 ? 8 : (UNI ? kUniMinBlocks : 4))
+    persistent_kernel(PersistentArgs a) {
+  static_assert(NT == kPersistentThreads || (NT == 128 && UNI), "128-thread CTAs: uniform geometry only");
+  static_assert(VAR == 0 || (UNI && !PACKED && NT == kPersistentThreads), "variants: uniform bytes, 256 threads");
   __shared__ VisitSmem sm;
   __shared__ uint16_t stash[(UNI || !PACKED) ? 1 : kStashWords];
   __shared__ uint32_t s_ord, s_quit, s_abort;
   __shared__ uint4 s_dec;   // the item's (m, k, bx, by), decoded by the ticket thread
   // Neighbour indices of the polls by a compare-and-wrap instead of the
   // modulo (measured with the per-thread ticket decode this kernel had
-  // before: 1.8 % faster on generic lattices at L = 4800, 0.8 % slower in the
-  // uniform build at L = 3200, which keeps the modulo).
-  constexpr bool kCmpWrap = !UNI;
+  // before: 1.8 % faster on generic lattices at L = 4800, 0.9 % in the
+  // 128-thread build at L = 6400, 0.8 % slower in the 256-thread uniform
+  // build at L = 3200, which keeps the modulo).
+  constexpr bool kCmpWrap = !(UNI && !PACKED && NT == kPersistentThreads && VAR == 0);
   // The uniform 256-thread build steps on the 8-byte-entry transition table
   // (rule8: one shared-memory read off the exchange path; L = 3200 -0.7 %,
   // -1.3 % at M = 1e-5 where more steps leave the exchange path).
-  constexpr bool kT8 = UNI;
+  constexpr bool kT8 = UNI && !PACKED && NT == kPersistentThreads && VAR == 0;
   // Generic builds: the epoch is released by a thread of the last warp, and
   // only warps 0 and 1 (the ticket thread and the pollers) meet at the top of
   // the loop, behind a named barrier, so that the release's wait for the
@@ -334,8 +342,43 @@ __global__ void __launch_bounds__(kPersistentThreads, UNI ? kUniMinBlocks : 4) p
       if (s_quit || s_abort) break;  // uniform across the CTA
       if (!early) decode();
       const uint32_t ord = s_ord;
-      if (UNI) {
-        visit_uniform_x0<kT8>(d, bx, by, m, sm);
+      if (VAR != 0) {
+        const int x0 = bx * kUniB, y0 = by * kUniB;
+        load_piece_uni(d, x0, y0, sm.tile, tid);
+        if (VAR & 2) corner_uni(d, x0, y0, sm.tile, tid, false);
+        __syncthreads();
+        const uint8_t* trans = reinterpret_cast<const uint8_t*>(sm.trans);
+        const bool edge = (VAR & 1) && (bx == 0 || bx == P - 1 || by == 0 || by == Py - 1);
+        if (edge)
+          fine_phases_var<(VAR & 2) != 0, true>(d, bx, by, m, sm.tile, sm.forder, trans);
+        else
+          fine_phases_var<(VAR & 2) != 0, false>(d, bx, by, m, sm.tile, sm.forder, trans);
+        store_piece_uni(d, x0, y0, sm.tile, tid);
+        if (VAR & 2) corner_uni(d, x0, y0, sm.tile, tid, true);
+      } else if (NT == 128) {
+        const int x0 = bx * kUniB, y0 = by * kUniB;
+        uint32_t rim_raw = 0;   // packed: the rim group of piece tid + 128
+        if (PACKED) {
+          load_piece_uni_packed(d, x0, y0, sm.tile, tid, d.bits);
+          rim_raw = load_piece_uni_packed(d, x0, y0, sm.tile, tid + 128, d.bits);
+        } else {
+          load_piece_uni(d, x0, y0, sm.tile, tid);
+          load_piece_uni(d, x0, y0, sm.tile, tid + 128);
+        }
+        __syncthreads();
+        own_fine_phases(d, bx, by, m, sm.tile, sm.forder, reinterpret_cast<const uint8_t*>(sm.trans));
+        if (PACKED) {
+          store_piece_uni_packed(d, x0, y0, sm.tile, tid, d.bits, 0u);
+          store_piece_uni_packed(d, x0, y0, sm.tile, tid + 128, d.bits, rim_raw);
+        } else {
+          store_piece_uni(d, x0, y0, sm.tile, tid);
+          store_piece_uni(d, x0, y0, sm.tile, tid + 128);
+        }
+      } else if (UNI) {
+        if (PACKED)
+          visit_uniform<false, PACKED>(d, bx, by, m, sm);
+        else
+          visit_uniform_x0<kT8>(d, bx, by, m, sm);
       } else {
         visit_generic<false, PACKED>(d, bx, by, m, sm, stash);
       }
@@ -343,7 +386,10 @@ __global__ void __launch_bounds__(kPersistentThreads, UNI ? kUniMinBlocks : 4) p
       if (log_point) {
         const int sV = slot_of(ord, colour ^ 2), sH = slot_of(ord, colour ^ 1),
                   sD = slot_of(ord, colour ^ 3);
-        if (UNI) {
+        if (NT == 128) {
+          count_pieces_uni<kUniSP, kColOff>(sm.tile, sm.hist, d.S, k, sV, sH, sD, tid);
+          count_pieces_uni<kUniSP, kColOff>(sm.tile, sm.hist, d.S, k, sV, sH, sD, tid + 128);
+        } else if (UNI) {
           count_visit_uni<kUniSP, kColOff>(sm.tile, sm.hist, d.S, k, sV, sH, sD);
         } else {
           count_visit_generic<PACKED>(d, bx, by, sm, k, sV, sH, sD);
@@ -1611,9 +1657,12 @@ bool resident_fits(const LatticeDesc& d, int device) {
 // Partitions with a 4-site segment (sides of 13 to 15 sites) run on the
 // one-byte image; every other lattice that fits runs on macros, whose image
 // is at most half as large.
+bool resident_on_macros(const LatticeDesc& d) {
+  return slot_axis_ok(d.ax) && slot_axis_ok(d.ay) && resident_layout(d, patch_planes(d)).bytes <= kResPatchBytes;
+}
+
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream) {
-  if (slot_axis_ok(a.d.ax) && slot_axis_ok(a.d.ay) &&
-      resident_layout(a.d, patch_planes(a.d)).bytes <= kResPatchBytes) {
+  if (resident_on_macros(a.d)) {
     const int bytes = resident_layout(a.d, patch_planes(a.d)).bytes;
     const void* fn = resident_patch_fn(a.d);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -1712,7 +1761,21 @@ cudaError_t launch_persistent(const PersistentArgs& args, int grid, cudaStream_t
   a.rcp_nb = div_rcp32(nb);
   a.rcp_per = div_rcp32(nb >> 2);
   a.rcp_half = div_rcp32((uint32_t)(a.d.P >> 1));
-  if (a.d.uniform64 && a.d.bits == 8)
+  if (flag_variant(a.d)) {
+    const int var = (a.d.nbh == 8 ? 2 : 0) | (a.d.reflect ? 1 : 0);
+    if (var == 1)
+      persistent_kernel<true, false, kPersistentThreads, 1><<<grid, kPersistentThreads, 0, stream>>>(a);
+    else if (var == 2)
+      persistent_kernel<true, false, kPersistentThreads, 2><<<grid, kPersistentThreads, 0, stream>>>(a);
+    else
+      persistent_kernel<true, false, kPersistentThreads, 3><<<grid, kPersistentThreads, 0, stream>>>(a);
+  } else if (a.threads == 128 && a.d.uniform64 && a.d.bits == 8)
+    persistent_kernel<true, false, 128><<<grid, 128, 0, stream>>>(a);
+  else if (a.threads == 128 && a.d.uniform64)
+    persistent_kernel<true, true, 128><<<grid, 128, 0, stream>>>(a);
+  else if (a.d.uniform64 && a.d.bits != 8)
+    persistent_kernel<true, true><<<grid, kPersistentThreads, 0, stream>>>(a);
+  else if (a.d.uniform64)
     persistent_kernel<true, false><<<grid, kPersistentThreads, 0, stream>>>(a);
   else if (a.d.bits != 8)
     persistent_kernel<false, true><<<grid, kPersistentThreads, 0, stream>>>(a);
@@ -1806,14 +1869,28 @@ cudaError_t launch_ll_merge(const LatticeDesc& d, const unsigned long long* ob, 
   return cudaGetLastError();
 }
 
+int persistent_grid128(int device) {
+  int sms = 0, per_sm = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  // the same grid for one byte and for 2 or 4 bits per site: the fewer CTAs
+  // of the two builds that an SM holds
+  int per_sm_packed = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel<true, false, 128>, 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_packed, persistent_kernel<true, true, 128>, 128, 0);
+  if (per_sm_packed < per_sm) per_sm = per_sm_packed;
+  if (per_sm > 8) per_sm = 8;
+  if (per_sm < 1) per_sm = 1;
+  return sms * per_sm;
+}
+
 int persistent_grid(int device, bool uniform) {
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (uniform) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel<true, false>, kPersistentThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel<true>, kPersistentThreads, 0);
     if (per_sm > kUniLaunchPerSM) per_sm = kUniLaunchPerSM;
   } else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel<false, false>, kPersistentThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel<false>, kPersistentThreads, 0);
   if (per_sm < 1) per_sm = 1;
   return sms * per_sm;
 }
