@@ -1293,7 +1293,10 @@ const char* escg_update_kernel(escg_t* h) {
 
 const char* escg_run_layout(escg_t* h, uint64_t n_mcs) {
   if (!h) return "";
-  const bool macros = h->use_resident ? resident_on_macros(h->desc) : (h->use_macro || h->use_group) && n_mcs >= h->macro_min;
+  // a resident launch to extinction ends at the next log point
+  const uint64_t launch = h->opt.stop_at_extinction ? std::min(n_mcs, (uint64_t)h->opt.log_every) : n_mcs;
+  const bool macros = h->use_resident ? resident_on_macros(h->desc, launch)
+                                      : (h->use_macro || h->use_group) && n_mcs >= h->macro_min;
   return macros ? "macros" : "bytes";
 }
 

@@ -129,8 +129,9 @@ cudaError_t launch_persistent_macro(const PersistentArgs& a, int grid, cudaStrea
 // Whole-lattice residency: one CTA runs MCS [m_begin, m_begin + n_mcs) with
 // the lattice in shared memory (counts of log points written in-kernel).
 bool resident_fits(const LatticeDesc& d, int device);
-// Whether it does so on macros (escg_resident_patch.cuh) or on the byte image.
-bool resident_on_macros(const LatticeDesc& d);
+// Whether a launch of n_mcs MCS does so on macros (escg_resident_patch.cuh) or
+// on the byte image.
+bool resident_on_macros(const LatticeDesc& d, uint64_t n_mcs);
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream);
 
 // Uniform geometry, boundary-mailbox variant (the default persistent path):

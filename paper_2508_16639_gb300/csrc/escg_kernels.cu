@@ -1655,14 +1655,22 @@ bool resident_fits(const LatticeDesc& d, int device) {
 }
 
 // Partitions with a 4-site segment (sides of 13 to 15 sites) run on the
-// one-byte image; every other lattice that fits runs on macros, whose image
-// is at most half as large.
-bool resident_on_macros(const LatticeDesc& d) {
-  return slot_axis_ok(d.ax) && slot_axis_ok(d.ay) && resident_layout(d, patch_planes(d)).bytes <= kResPatchBytes;
+// one-byte image, and so do short launches past 16384 sites, where the macros'
+// image and tables take longer to make than a few MCS win back.  us per MCS of
+// launches of n MCS, byte image and macros: L = 160 n = 1 33.4, 44.7, n = 2 29.3, 30.8,
+// n = 3 1.07 x; S = 5 33.5, 46.8 / 29.4, 33.0 / 28.0, 28.1; 191 43.9, 55.5 / 39.8, 40.2;
+// packed rows, read bit by bit, meet at 3 (2 bits) and 4.  Up to 128 x 128 n = 1 gains
+// (L = 100 37.3, 24.9).  Every other lattice that fits runs on macros, whose image is
+// at most half as large.
+bool resident_on_macros(const LatticeDesc& d, uint64_t n_mcs) {
+  if (!slot_axis_ok(d.ax) || !slot_axis_ok(d.ay)) return false;
+  const int planes = patch_planes(d);
+  if (resident_layout(d, planes).bytes > kResPatchBytes) return false;
+  return (int64_t)d.L * d.H <= 16384 || n_mcs >= (uint64_t)(planes + (d.bits == 8 ? 1 : 2));
 }
 
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream) {
-  if (resident_on_macros(a.d)) {
+  if (resident_on_macros(a.d, a.n_mcs)) {
     const int bytes = resident_layout(a.d, patch_planes(a.d)).bytes;
     const void* fn = resident_patch_fn(a.d);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -99,3 +99,26 @@ def test_few_exchanges_move_the_line():
         o, _ = O.replay_run(O.init(256, 5, 0.0, 1), D, 1.0, 1.0, X, 1, 17)
         assert np.array_equal(g.snapshot(), o)
         g.close()
+
+
+@pytest.mark.parametrize("L,H,S,kw,line", [(128, 127, 3, {}, 1), (130, 129, 3, {}, 2), (191, 160, 5, {}, 3),
+                                           (160, 150, 3, dict(bits_per_site=2), 3), (160, 150, 5, dict(bits_per_site=4), 4),
+                                           (300, 270, 3, dict(persistent=4, reflecting_boundary=True), 2)])
+def test_resident_launches(L, H, S, kw, line):
+    """The same line for whole-lattice residency, launch by launch."""
+    D = O.circulant(S, (1,) if S == 3 else (1, 2))
+    rule = dict(reflect=kw.get("reflecting_boundary", False))
+    for stop in (False, True):
+        g = E.Lattice(L, S, D, (1.0, 1.0, 2.0), 5, p_empty=0.2, H=H, log_every=5, stop_at_extinction=stop, **kw)
+        assert g.update_kernel == "resident_kernel" and _line(g) == line
+        lat, m = O.init(L, S, 0.2, 5, H=H), 0
+        first = lat
+        for n in (1, line, 2, 9, 1, 13):
+            g.run(n)
+            lat, _ = O.replay_run(lat, D, 1.0, 1.0, 2.0, 5, n, mcs_begin=m, **rule)
+            m += n
+            assert np.array_equal(g.snapshot(), lat), m
+        _, log = g.counts_log()
+        _, olog, _ = O.run_observed(first, D, 1.0, 1.0, 2.0, 5, m, log_every=5, **rule)
+        assert np.array_equal(log, olog) and g.mcs == m
+        g.close()
