@@ -72,3 +72,28 @@ def test_graphs_are_built_once(chunks, builds):
     assert srv.graph_builds == builds
     for rid, sp in zip(ids, specs):
         _check(srv, rid, sp)
+
+
+@pytest.mark.parametrize("n", [20, 200, 320])
+def test_small_replicas_stop_at_extinction(n):
+    """Replicas of 2 x 2 blocks alone (resident: one or two to an SM) stop at the
+    log point where one species is left, each for itself; a lattice that starts
+    with one never runs."""
+    sides = (8, 9, 10, 11, 12, 16, 17, 18)   # 13 to 15 have 4-site segments and stay in the chunk kernel
+    specs = [_spec(sides[i % 8], 100 + i, 60 + i % 7, S=3 if i % 2 else 5, stop=i % 4 != 3, X=0.5,
+                   p_empty=1.0 if i % 19 == 5 else 0.6) for i in range(n)]
+    b = E.Batch(specs, log_every=5)
+    b.run(10).run()
+    assert (b.threads == 0) == (n <= 200) and b.active == 0   # 320: more than two to an SM
+    mcs, ext, counts = b.status()
+    seen = set()
+    for i, sp in enumerate(specs):
+        lat, log, mend = O.run_observed(O.init(sp["L"], sp["S"], sp["p_empty"], sp["seed"]), sp["digraph"], *sp["rates"],
+                                        sp["seed"], sp["max_mcs"], log_every=5, stop_at_extinction=sp["stop_at_extinction"])
+        alive = int((log[-1][1:] > 0).sum())
+        assert mcs[i] == mend and np.array_equal(b.snapshot(i), lat), i
+        assert np.array_equal(counts[i, :sp["S"] + 1], log[-1]), i
+        assert bool(ext[i]) == (sp["stop_at_extinction"] and alive <= 1), i
+        seen.add((mend == 0, 0 < mend < sp["max_mcs"], mend == sp["max_mcs"]))
+    assert len(seen) == 3
+    b.close()
