@@ -533,11 +533,6 @@ __device__ __forceinline__ void patch_item_run(typename MacroOf<PL>::type* __res
 
 // ---------------------------------------------------------------------------
 // One axis of a partition by slots (segments of 2 or 3 sites).
-struct SlotAxis {
-  AxisGeom g;
-  int P, G, n;   // coarse blocks, fine segments, sites
-};
-
 __host__ __device__ inline bool slot_axis_ok(const AxisGeom& g) {
   // all segments 2 or 3 sites wide
   const bool a = g.r == 0 || (g.Qa > 0 && g.fqa >= 2 && g.fqa + (g.fra > 0 ? 1 : 0) <= 3);
@@ -594,13 +589,6 @@ __host__ __device__ inline void axis_quad(const AxisGeom& g, int P, int k2, int&
   const int irr = a ? ia : ib;
   pos = q >= irr ? na * (ha - ia) + (i - na) * (hb - ib) + (q - irr) : regular + na * ia + (i - na) * ib + q;
 }
-
-// Reciprocal of quot_rcp (0: d = 1, no division).
-__host__ __device__ inline uint32_t quot_rcp_of(int d) { return d <= 1 ? 0u : 0xFFFFFFFFu / (uint32_t)d + 1u; }
-// floor(n / d) for n d < 2^32 from ceil(2^32 / d) (0 for d = 1): the product
-// overshoots n / d by less than n / 2^32 < 1 / d.
-__device__ __forceinline__ uint32_t quot_rcp(uint32_t n, uint32_t rcp) { return rcp ? __umulhi(n, rcp) : n; }
-
 
 // First joint slot of block b of an axis, and its slots up to the next block's.
 __host__ __device__ inline int block_slot(const AxisGeom& g, int b) {
