@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 8 : 4)
           __threadfence();
           if (atomicAdd(&st->pend[ring], 1u) == nb - 1u) {
             // last block of this log point: every contribution is in acc
+            // (flag_log in line: a call of it costs L = 3200 1 %)
             __threadfence();
             unsigned long long c[kMaxStates], rest = (unsigned long long)d.L * (unsigned long long)d.H;
             for (int v = 1; v < kMaxStates; ++v) {
@@ -586,7 +587,7 @@ __device__ __forceinline__ uint32_t macro_unpack4(uint32_t v) {
 
 template <int PL>
 __global__ void __launch_bounds__(256) macro_fill_kernel(LatticeDesc d, typename MacroOf<PL>::type* G, RunState* st) {
-  if (macro_fill_off(st)) return;
+  const bool off = macro_fill_off(st);   // asked for before the stores: its load must not hold the others up
   const int nt = d.L >> 4, rows = d.H >> 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x, ky = blockIdx.y * blockDim.y + threadIdx.y;
   if (t >= nt || ky >= rows) return;
@@ -601,6 +602,7 @@ __global__ void __launch_bounds__(256) macro_fill_kernel(LatticeDesc d, typename
                        ((uint64_t)macro_pack4<PL>(w.z) << (16 * PL)) | ((uint64_t)macro_pack4<PL>(w.w) << (24 * PL));
     line[h] = (p << (2 * PL)) | prev;
   }
+  if (off) return;
   uint8_t* out = reinterpret_cast<uint8_t*>(G + (size_t)ky * d.GQ + 8 * t);
   if (PL == 1) {
     // nibble i of each row -> byte i
@@ -628,7 +630,7 @@ __global__ void __launch_bounds__(256) macro_fill_kernel(LatticeDesc d, typename
 template <int PL>
 __global__ void __launch_bounds__(256) macro_drain_kernel(LatticeDesc d, const typename MacroOf<PL>::type* G,
                                                          const RunState* st) {
-  if (!st->on_macros) return;
+  const bool on = st->on_macros != 0u;
   const int nt = d.L >> 4, rows = d.H >> 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x, ky = blockIdx.y * blockDim.y + threadIdx.y;
   if (t >= nt || ky >= rows) return;
@@ -657,6 +659,7 @@ __global__ void __launch_bounds__(256) macro_drain_kernel(LatticeDesc d, const t
       line[h] = (uint64_t)__byte_perm(m.x, m.y, sel) | ((uint64_t)__byte_perm(m.z, m.w, sel) << 32);
     }
   }
+  if (!on) return;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     // drop site 16 t - 1, append site 16 t + 15

@@ -573,7 +573,7 @@ constexpr int kConvRows = 64;
 template <int PL>
 __global__ void __launch_bounds__(256)
     macro_fill_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, typename MacroOf<PL>::type* G, RunState* st) {
-  if (macro_fill_off(st)) return;
+  const bool off = macro_fill_off(st);
   typedef typename MacroOf<PL>::type MT;
   __shared__ int2 rows[kConvRows];
   const int x = blockIdx.x * 32 + threadIdx.x, y0 = blockIdx.y * kConvRows, t = threadIdx.y * 32 + threadIdx.x;
@@ -592,8 +592,9 @@ __global__ void __launch_bounds__(256)
   for (int k = threadIdx.y; k < kConvRows; k += 8) {
     if (y0 + k >= nsy) break;
     const int2 r = rows[k];
-    G[(size_t)(y0 + k) * gpitch + x] = (MT)(site(r.x, c.x) | (site(r.x, c.y) << (2 * PL)) | (site(r.y, c.x) << (4 * PL)) |
-                                            (site(r.y, c.y) << (6 * PL)));
+    const MT v = (MT)(site(r.x, c.x) | (site(r.x, c.y) << (2 * PL)) | (site(r.y, c.x) << (4 * PL)) |
+                      (site(r.y, c.y) << (6 * PL)));
+    if (!off) G[(size_t)(y0 + k) * gpitch + x] = v;
   }
 }
 
@@ -601,7 +602,7 @@ template <int PL>
 __global__ void __launch_bounds__(256)
     macro_drain_any_kernel(LatticeDesc d, int nsx, int nsy, int gpitch, const typename MacroOf<PL>::type* G,
                            const RunState* st) {
-  if (!st->on_macros) return;
+  const bool on = st->on_macros != 0u;
   __shared__ int rows[kConvRows];
   const int c0 = 4 * (blockIdx.x * 32 + threadIdx.x), y0 = blockIdx.y * kConvRows, t = threadIdx.y * 32 + threadIdx.x;
   if (t < kConvRows && y0 + t < d.H) rows[t] = site_slot(d.ay, nsy, y0 + t);
@@ -621,6 +622,7 @@ __global__ void __launch_bounds__(256)
     for (int e = 0; e < 4; ++e)
       if (mx[e] >= 0)
         u |= (((uint32_t)row[mx[e] >> 1] >> (2 * PL * (2 * (my & 1) + (mx[e] & 1)))) & (PL == 1 ? 3u : 15u)) << (8 * e);
+    if (!on) break;
     uint8_t* out = d.lat + (size_t)y * d.pitch;
     if (d.bits == 8 && c0 + 4 > d.L) {   // no row padding written
       for (int e = 0; c0 + e < d.L; ++e) out[c0 + e] = (uint8_t)(u >> (8 * e));
