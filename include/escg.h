@@ -159,10 +159,19 @@ typedef struct {
                                     through a byte image allocated on first
                                     use).  Results are identical for all three;
                                     the device buffer is H rows of
-                                    escg_lattice_pitch_ex(L, b) bytes.        */
+                                    escg_lattice_pitch_ex(L, b) bytes.
+                                    A handle whose calls run on macros (see
+                                    escg_run_layout) keeps one more array on
+                                    the device for its life: about L*H/4 bytes
+                                    with S <= 3 and certain edges, else L*H/2 --
+                                    as much again as a packed lattice, twice as
+                                    much for 2 bits with uncertain edges.
+                                    Without room for it, or in persistent = 0,
+                                    2 and 6, the lattice alone is kept.       */
     int32_t autotune;            /* 1 (with persistent = 1): on the first
                                     handle of its (device, L, H, S,
-                                    bits_per_site, neighbourhood, boundary),
+                                    bits_per_site, neighbourhood, boundary,
+                                    certain edges or not),
                                     time every distinct launch mode and CTA
                                     count on a copy of the initial lattice
                                     (10 MCS of warm-up, 20 timed) and keep the

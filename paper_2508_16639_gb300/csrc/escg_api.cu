@@ -457,9 +457,9 @@ int ensure_records(escg* h, size_t words) {
   return ESCG_OK;
 }
 
-// The macro array of the flag kernel, a quarter of the one-byte lattice (half
-// with 4 bits per site), allocated on first use; false if there is no room
-// (the flag kernel then works on the lattice array itself).
+// The macro array, a quarter of the one-byte lattice (half with 4 bits per site),
+// allocated with the selection that uses it; false if there is no room (the
+// kernels on bytes then run).
 bool ensure_macros(escg* h) {
   if (h->d_macros) return true;
   if (cudaMalloc(&h->d_macros, macro_bytes(h->desc)) == cudaSuccess) return true;
@@ -558,8 +558,9 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
   // Whole-lattice residency: on request (4), and by default (1) for a generic
   // partition with 2 x 2 coarse blocks (L, H < 192 and not 128), where it was
   // measured 1.4-2.2x faster than the flag kernel's dependency chain of
-  // generic visits (tied at L = 200, slower beyond; the mailbox kernel is
-  // faster for the uniform L = 128).
+  // generic visits (tied at L = 200, slower beyond).  The uniform L = 128 stays
+  // with the mailbox kernel, which was faster than the byte image (13.6 us per
+  // MCS; residency on macros takes 10.3).
   if ((persistent == 4 || (persistent == 1 && !d.uniform64 && p.P == 2 && py.P == 2)) &&
       resident_fits(d, h->device)) {
     h->use_resident = true;
@@ -602,6 +603,10 @@ int select_kernel(escg* h, int persistent, int ctas_per_sm) {
       h->grid = grid;
       h->flag_threads = threads;
     }
+  }
+  if (!h->use_macro && !h->use_group && h->d_macros) {   // of a candidate that the tuner did not take
+    cudaFree(h->d_macros);
+    h->d_macros = nullptr;
   }
   h->macro_min = h->use_macro || h->use_group ? macro_min_mcs(d, h->use_group, h->flag_threads == 128) : 1;
   if (ctas_per_sm > 0) {
