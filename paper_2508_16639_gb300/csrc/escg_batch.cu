@@ -1555,11 +1555,13 @@ int engine_run(Engine* e, uint64_t chunks, bool until_idle) {
 }
 
 int engine_check(Engine* e) {
-  if (e->settled) return ESCG_OK;
+  if (e->settled && e->own_stream) return ESCG_OK;
+  // a caller's stream may hold the caller's work too
   if (cudaStreamSynchronize(e->stream) != cudaSuccess) {
     set_last_error("engine stream failed: %s", cudaGetErrorString(cudaGetLastError()));
     return ESCG_ECUDA;
   }
+  if (e->settled) return ESCG_OK;
   BatchCtl ctl;
   if (cudaMemcpy(&ctl, e->d_ctl, sizeof ctl, cudaMemcpyDeviceToHost) != cudaSuccess) return ESCG_ECUDA;
   if (ctl.error & kErrTimeout) {

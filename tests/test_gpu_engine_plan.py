@@ -97,3 +97,23 @@ def test_small_replicas_stop_at_extinction(n):
         seen.add((mend == 0, 0 < mend < sp["max_mcs"], mend == sp["max_mcs"]))
     assert len(seen) == 3
     b.close()
+
+
+def test_sync_waits_for_the_callers_stream():
+    """sync, status and snapshot wait for what the caller has put on the stream of a
+    batch, also when the batch has nothing of its own there."""
+    torch = pytest.importorskip("torch")
+    st = torch.cuda.Stream()
+    b = E.Batch([_spec(64, 1, 20), _spec(200, 2, 20)], stream=st)
+    b.run()
+    b.sync()
+    for call in (b.sync, b.status, lambda: b.snapshot(1)):
+        with torch.cuda.stream(st):
+            torch.cuda._sleep(20_000_000)   # about 10 ms
+            ev = torch.cuda.Event()
+            ev.record(st)
+        call()
+        assert ev.query()
+    o, _ = O.replay_run(O.init(200, 3, 0.25, 2), O.circulant(3, (1,)), 1.0, 1.0, 2.0, 2, 20)
+    assert np.array_equal(b.snapshot(1), o)
+    b.close()
