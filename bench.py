@@ -60,20 +60,21 @@ UNIT = "site-updates/s"
 # table lookup are memory instructions and not counted.
 ALG_INT_INSTR_PER_ATTEMPT = 24
 
-# DRAM traffic of persistent_kernel from one ncu capture (bytes per launch of
-# a 10-MCS chunk at L = 3200), valid only for that kernel and workload and the
-# kernel sources it was taken from (hash below); None otherwise.
-NCU_TRAFFIC = {"sources_sha1": "f3d15f12ffa514d9d6328dec9a3d032ff0fde2ee", "bytes_per_launch": 10304768 + 817493,
-               "kernel": "persistent_kernel", "L": 3200, "mcs_per_launch": 10,
-               "profile": "profiles/persistent_kernel_L3200_M1e-4.md"}
+# DRAM traffic of a 10-MCS call at L = 3200 from one ncu capture (bytes read and
+# written of the conversion into macros, the flag kernel on macros and the
+# conversion back), valid only for that kernel and workload and the kernel
+# sources it was taken from (hash below); None otherwise.
+NCU_TRAFFIC = {"sources_sha1": "57dfa2d4728a21276cc93db0b8a6f529460cd89d", "bytes_per_launch": 10250496 + 3912448 + 519936 + 2566912,
+               "kernel": "persistent_kernel", "layout": "macros", "L": 3200, "mcs_per_launch": 10,
+               "profile": "profiles/macro_kernels_counters.md"}
 
 
-KERNEL_SOURCES = ("escg_kernels.cu", "escg_device.cuh", "escg_types.h", "escg_internal.h", "escg_tma.cuh",
-                  "escg_resident.cuh")
+KERNEL_SOURCES = ("escg_flag.cu", "escg_patch.cuh", "escg_sync.cuh", "escg_device.cuh", "escg_types.h",
+                  "escg_internal.h")
 
 
 def _sources_sha1() -> str:
-    """Hash of the translation unit that defines the single-lattice kernels."""
+    """Hash of the translation unit that defines the flag kernel on macros."""
     h = hashlib.sha1()
     csrc = os.path.join(ROOT, "paper_2508_16639_gb300", "csrc")
     for fn in KERNEL_SOURCES:
@@ -753,11 +754,11 @@ def main():
     achieved = per_launch_attempts * ALG_INT_INSTR_PER_ATTEMPT / avg_launch_s
     traffic = (NCU_TRAFFIC["bytes_per_launch"]
                if (NCU_TRAFFIC["sources_sha1"] == _sources_sha1() and g.update_kernel == NCU_TRAFFIC["kernel"]
-                   and w.L == NCU_TRAFFIC["L"] and mps == NCU_TRAFFIC["mcs_per_launch"]) else None)
+                   and g.run_layout(mps) == NCU_TRAFFIC["layout"] and w.L == NCU_TRAFFIC["L"] and mps == NCU_TRAFFIC["mcs_per_launch"]) else None)
     tile_gbs = 2.0 * per_launch_attempts / avg_launch_s / 1e9
     l2_peak = E.l2_copy_gbs(N, 200)
     hbm_peak, hbm_src = _hbm_peak()
-    roofline = {"bound": "alu", "kernel": g.update_kernel,
+    roofline = {"bound": "alu", "kernel": g.update_kernel, "layout": g.run_layout(mps),
                 "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tinstr/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "alg_int_instr_per_attempt": ALG_INT_INSTR_PER_ATTEMPT,

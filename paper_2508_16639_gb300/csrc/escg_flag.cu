@@ -117,7 +117,7 @@ static __device__ __noinline__ void flag_log(RunState* st, const PersistentArgs&
 }
 
 // Bound by the colour chain while a phase is one wave (L = 3200: issue active
-// 52 %, 37 executed thread instructions per attempt where the byte tile took
+// 52 %, 39 executed thread instructions per attempt where the byte tile took
 // 52), by integer issue once phases are several waves deep.  us per MCS of
 // 10-MCS launches, conversions included, against the byte tile: L = 3200 23.2 ->
 // 19.2 (4.4e11 -> 5.3e11 site updates/s), Moore 24.5 -> 19.9, L = 12800 304 ->
@@ -383,7 +383,7 @@ __device__ __noinline__ void any_count(AnySmem<PL>& sm, int xoff, int ncx, int n
 // a phase's words are drawn before the barrier that ends the one before.  us per
 // MCS against the byte tile, 10-MCS counts, M = 1e-4: L = 4800 114.6 -> 90.9 (2.0e11
 // -> 2.5e11 site updates/s), 12700 619 -> 406, Moore 115.1 -> 93.8, reflecting 127.6 ->
-// 110.9, 6400 x 1600 45.9 -> 35.2; at 2 bits per site 193 -> 93.7, at 4 193 -> 118; S = 5,
+// 107.8, 6400 x 1600 45.9 -> 35.2; at 2 bits per site 193 -> 93.7, at 4 193 -> 118; S = 5,
 // L = 12700 619 -> 478, 8000 287 -> 278, 4800 114.6 -> 115.4 (bytes kept).
 template <int PL, int LG, bool REFLECT>
 __global__ void __launch_bounds__(256, 4) persistent_macro_any_kernel(const __grid_constant__ PersistentArgs a, int nsx,
@@ -730,8 +730,9 @@ int persistent_macro_any_grid(const LatticeDesc& d, int device) {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, macro_any_fn(d), 256, 0) != cudaSuccess) return 0;
   const int grid = sms * (occ < 4 ? occ : 4);
   // Where it beats the flag kernel on bytes: with 2 bits per site (S <= 3), the
-  // reflecting boundary only once a phase is two waves deep (its mirrored steps
-  // lengthen the chain: L = 800, Moore, 44.1 -> 52.5 us per MCS); with 4 bits only
+  // reflecting boundary only once a phase is two waves deep (mirrored steps
+  // lengthened the chain, L = 800, Moore, 44.1 -> 52.5 us per MCS, before their
+  // entries came from a table; not measured since); with 4 bits only
   // past half of the L2, where the bytes no longer stay.  Packed lattices, whose
   // byte tiles cost a conversion each way, always.
   if (d.bits == 8) {

@@ -669,8 +669,9 @@ static int fine_rows(const LatticeDesc& d) { return d.ay.r * d.ay.Qa + (d.Py - d
 //  * Moore, periodic: L = 400 18.1 (39.5), S = 5 26.3 (40.4); 64 x 64 blocks, L =
 //    1024, against the flag kernel on macros 12.5 (15.5), S = 5 13.7 (17.9); two
 //    CTAs per SM, 2 bits per site: 1600 28.7 (40.8), 2200 26.9 (39.2).
-//  * reflecting on 64 x 64 blocks, L = 1024: 13.4 (22.2), S = 5 15.2.  With 3-site
-//    segments the mirrored steps are slower: L = 800 35.0 (28.2), not built.
+//  * reflecting on 64 x 64 blocks, L = 1024: 12.9 (22.2), S = 5 13.9.  With 3-site
+//    segments the mirrored steps were slower, L = 800 35.0 (28.2), before their
+//    entries came from a table (not measured since): not built.
 //  * 64 x 64 blocks, von Neumann, periodic: L = 1024 12.5 (12.6), 1536 12.3 (11.9):
 //    not built.
 static const void* group_fn(const LatticeDesc& d, int groups) {
