@@ -64,7 +64,7 @@ ALG_INT_INSTR_PER_ATTEMPT = 24
 # written of the conversion into macros, the flag kernel on macros and the
 # conversion back), valid only for that kernel and workload and the kernel
 # sources it was taken from (hash below); None otherwise.
-NCU_TRAFFIC = {"sources_sha1": "57dfa2d4728a21276cc93db0b8a6f529460cd89d", "bytes_per_launch": 10250496 + 3912448 + 519936 + 2566912,
+NCU_TRAFFIC = {"sources_sha1": "e81fb76f4b32701143e75cf3b22415ddbf0247d4", "bytes_per_launch": 10250496 + 3912448 + 519936 + 2566912,
                "kernel": "persistent_kernel", "layout": "macros", "L": 3200, "mcs_per_launch": 10,
                "profile": "profiles/macro_kernels_counters.md"}
 

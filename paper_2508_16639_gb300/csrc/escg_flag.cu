@@ -755,8 +755,9 @@ int persistent_macro_grid(const LatticeDesc& d, int device, int threads) {
 // macros win back at some us per MCS.  Calls below the lines run on bytes.  us per
 // MCS of calls of n MCS on bytes and on macros (M = 1e-4 unless stated), the line
 // where they meet:
-//  * owners: L = 800 n = 1 40.4, 47.5, n = 2 31.7, 32.4, n = 5 26.8, 23.5; L = 2200 Moore
-//    53.5, 64.9 / 45.0, 45.7 / 40.5, 33.8.  On 64 x 64 blocks with a reflecting
+//  * owners: L = 800 n = 1 40.4, 47.5, n = 2 31.7, 33.2, n = 3 29.1, 28.5, n = 5 26.8, 23.5;
+//    L = 400 n = 2 33.7, 31.8; L = 2200 Moore 53.5, 64.9 / 45.0, 46.4 / 43.4, 40.0, L = 1600
+//    n = 2 48.3, 45.4.  On 64 x 64 blocks with a reflecting
 //    boundary n = 1 already gains (L = 1024 1.15 x).
 //  * flags, 64 x 64 blocks, 2 bits per site: L = 3200 34.1, 39.6 / 29.4, 29.1 / 25.3,
 //    22.7; the Moore bytes are slower and meet at 1 (39.3, 40.5), deep phases (L = 6400)
@@ -770,9 +771,12 @@ int persistent_macro_grid(const LatticeDesc& d, int device, int threads) {
 //    624, 540.
 uint32_t macro_min_mcs(const LatticeDesc& d, bool group, bool deep) {
   const bool one = patch_planes(d) == 1, moore = d.nbh == 8, refl = d.reflect != 0;
-  if (group) return d.blocks64 && refl ? 1u : 2u;
-  if (!d.blocks64) return d.bits != 8 ? 1u : ((size_t)d.H * d.L >= (32u << 20) ? 2u : 3u);
   const bool few = d.tx < 0x80000000u;   // fewer than half the attempts exchange
+  if (group) {
+    if (d.blocks64 && refl) return 1u;
+    return !few && (size_t)d.H * d.L > (moore ? 1u << 22 : 1u << 18) ? 3u : 2u;
+  }
+  if (!d.blocks64) return d.bits != 8 ? 1u : ((size_t)d.H * d.L >= (32u << 20) ? 2u : 3u);
   if (d.bits != 8) {
     if (moore || refl) return 1u;
     return one ? (deep ? 1u : 2u) : (few ? 5u : (deep ? 2u : 3u));

@@ -52,6 +52,7 @@ CASES = [
     (400, 530, 3, dict(persistent=3, neighbourhood=8), None, 3),
     (400, 400, 3, dict(persistent=3, bits_per_site=2), None, 1),
     (400, 400, 3, {}, None, 2),                                    # owners, beside the byte owners
+    (600, 450, 3, {}, None, 3),
     (400, 400, 5, dict(neighbourhood=8), None, 2),                 # beside the flags
     (384, 512, 3, dict(neighbourhood=8), None, 2),
     (384, 512, 5, dict(reflecting_boundary=True), None, 1),
