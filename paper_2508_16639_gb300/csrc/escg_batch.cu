@@ -1067,8 +1067,8 @@ struct Engine {
   int grid_tma[3] = {0, 0, 0};
   std::vector<SlotUpload> up;     // replicas added and not yet on the device (at most kUpload)
   std::vector<CUtensorMap> up_maps;
-  SlotUpload* d_up = nullptr;
-  static constexpr size_t kUpload = 4096;   // bounds the staging memory (11 MB)
+  SlotUpload* d_up = nullptr;     // their staging, behind the arena
+  static constexpr size_t kUpload = 512;   // bounds the staging memory (1.4 MB)
   int fail_uploads = 0;           // test hook: uploads that fail before they begin
   bool settled = false;           // no work enqueued since the last engine_check
   uint32_t* h_pinned = nullptr;   // pinned host words (admit list staging, counters)
@@ -1158,11 +1158,8 @@ void engine_free(Engine* e) {
   cudaFree(e->d_states);
   cudaFree(e->d_ctl);
   cudaFree(e->d_active);
-  cudaFree(e->d_active_tmp);
   cudaFree(e->d_table);
-  cudaFree(e->d_admit);
   cudaFree(e->d_maps);
-  cudaFree(e->d_up);
   if (e->h_pinned) cudaFreeHost(e->h_pinned);
   if (e->own_stream && e->stream) cudaStreamDestroy(e->stream);
   e->arena_mem = nullptr;
@@ -1189,17 +1186,22 @@ int engine_init(Engine* e, int max_slots, size_t arena_bytes, size_t table_cap, 
       e->own_stream = true;
     }
   }
-  if (err == cudaSuccess) err = cudaMalloc(&e->arena_mem, arena_bytes);
+  // the arena and behind it the staging of uploads; the lists (active, its next,
+  // the admissions) together too: every allocation is 10 to 30 us of a creation
+  const size_t stage = align_up(arena_bytes, 256);
+  if (err == cudaSuccess)
+    err = cudaMalloc(&e->arena_mem, stage + sizeof(SlotUpload) * std::min<size_t>((size_t)max_slots, Engine::kUpload));
+  if (err == cudaSuccess) e->d_up = reinterpret_cast<SlotUpload*>(e->arena_mem + stage);
   if (err == cudaSuccess) err = cudaMalloc(&e->d_slots, sizeof(SlotDesc) * max_slots);
   if (err == cudaSuccess) err = cudaMalloc(&e->d_states, sizeof(SlotState) * max_slots);
   if (err == cudaSuccess) err = cudaMalloc(&e->d_ctl, sizeof(BatchCtl));
-  if (err == cudaSuccess) err = cudaMalloc(&e->d_active, sizeof(uint32_t) * max_slots);
-  if (err == cudaSuccess) err = cudaMalloc(&e->d_active_tmp, sizeof(uint32_t) * max_slots);
+  if (err == cudaSuccess) err = cudaMalloc(&e->d_active, sizeof(uint32_t) * (3 * (size_t)max_slots + 1));
+  if (err == cudaSuccess) {
+    e->d_active_tmp = e->d_active + max_slots;
+    e->d_admit = e->d_active_tmp + max_slots;
+  }
   if (err == cudaSuccess) err = cudaMalloc(&e->d_table, sizeof(uint32_t) * table_cap);
-  if (err == cudaSuccess) err = cudaMalloc(&e->d_admit, sizeof(uint32_t) * (max_slots + 1));
   if (err == cudaSuccess) err = cudaMalloc(&e->d_maps, sizeof(CUtensorMap) * max_slots);
-  if (err == cudaSuccess)
-    err = cudaMalloc(&e->d_up, sizeof(SlotUpload) * std::min<size_t>((size_t)max_slots, Engine::kUpload));
   if (err == cudaSuccess) err = cudaMallocHost(&e->h_pinned, sizeof(uint32_t) * (max_slots + 16));
   if (err == cudaSuccess) err = cudaMemsetAsync(e->d_ctl, 0, sizeof(BatchCtl), e->stream);
   if (err == cudaSuccess) err = cudaMemsetAsync(e->d_states, 0, sizeof(SlotState) * max_slots, e->stream);
@@ -1360,10 +1362,9 @@ int engine_upload(Engine* e) {
   size_t groups = 0;   // of 4 sites, of the largest
   for (const SlotUpload& u : e->up) groups = std::max(groups, (size_t)u.sd.d.H * (size_t)u.sd.d.pitch / 4);
   const unsigned per = (unsigned)std::min<size_t>(std::max<size_t>((groups + 2047) / 2048, 1), 1024);
-  for (size_t i = 0; i < n && err == cudaSuccess; i += 32768) {   // grid limit in y
-    const unsigned ny = (unsigned)std::min<size_t>(n - i, 32768);
-    batch_place_kernel<<<ny, 128, 0, e->stream>>>(e->d_up + i, e->d_slots, e->d_states);
-    batch_init_kernel<<<dim3(per, ny), 256, 0, e->stream>>>(e->d_up + i, e->d_states);
+  if (err == cudaSuccess) {
+    batch_place_kernel<<<(unsigned)n, 128, 0, e->stream>>>(e->d_up, e->d_slots, e->d_states);
+    batch_init_kernel<<<dim3(per, (unsigned)n), 256, 0, e->stream>>>(e->d_up, e->d_states);
     err = cudaGetLastError();
     e->launches += 2;
   }

@@ -1,4 +1,4 @@
-"""Set-up of the engine's replicas: in groups of 4096, and again after a failure."""
+"""Set-up of the engine's replicas: in groups, and again after a failure."""
 import numpy as np
 import pytest
 
