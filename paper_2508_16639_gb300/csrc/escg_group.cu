@@ -581,6 +581,7 @@ __global__ void __launch_bounds__(256)
   __syncthreads();
   if (x >= nsx) return;
   const int2 c = slot_sites(d.ax, d.L, x);
+  if (off) return;   // asked for above: its load passes beside the divisions
   auto site = [&](int row, int col) -> uint32_t {
     if (row < 0 || col < 0) return 0u;
     const uint8_t* p = d.lat + (size_t)row * d.pitch;
@@ -592,9 +593,8 @@ __global__ void __launch_bounds__(256)
   for (int k = threadIdx.y; k < kConvRows; k += 8) {
     if (y0 + k >= nsy) break;
     const int2 r = rows[k];
-    const MT v = (MT)(site(r.x, c.x) | (site(r.x, c.y) << (2 * PL)) | (site(r.y, c.x) << (4 * PL)) |
-                      (site(r.y, c.y) << (6 * PL)));
-    if (!off) G[(size_t)(y0 + k) * gpitch + x] = v;
+    G[(size_t)(y0 + k) * gpitch + x] = (MT)(site(r.x, c.x) | (site(r.x, c.y) << (2 * PL)) | (site(r.y, c.x) << (4 * PL)) |
+                                            (site(r.y, c.y) << (6 * PL)));
   }
 }
 
@@ -611,6 +611,7 @@ __global__ void __launch_bounds__(256)
   int mx[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) mx[e] = c0 + e < d.L ? site_slot(d.ax, nsx, c0 + e) : -1;
+  if (!on) return;
 #pragma unroll 4
   for (int k = threadIdx.y; k < kConvRows; k += 8) {
     const int y = y0 + k;
@@ -622,7 +623,6 @@ __global__ void __launch_bounds__(256)
     for (int e = 0; e < 4; ++e)
       if (mx[e] >= 0)
         u |= (((uint32_t)row[mx[e] >> 1] >> (2 * PL * (2 * (my & 1) + (mx[e] & 1)))) & (PL == 1 ? 3u : 15u)) << (8 * e);
-    if (!on) break;
     uint8_t* out = d.lat + (size_t)y * d.pitch;
     if (d.bits == 8 && c0 + 4 > d.L) {   // no row padding written
       for (int e = 0; c0 + e < d.L; ++e) out[c0 + e] = (uint8_t)(u >> (8 * e));
