@@ -1659,14 +1659,16 @@ bool resident_fits(const LatticeDesc& d, int device) {
 // image and tables take longer to make than a few MCS win back.  us per MCS of
 // launches of n MCS, byte image and macros: L = 160 n = 1 33.4, 44.7, n = 2 29.3, 30.8,
 // n = 3 1.07 x; S = 5 33.5, 46.8 / 29.4, 33.0 / 28.0, 28.1; 191 43.9, 55.5 / 39.8, 40.2;
-// packed rows, read bit by bit, meet at 3 (2 bits) and 4.  Up to 128 x 128 n = 1 gains
-// (L = 100 37.3, 24.9).  Every other lattice that fits runs on macros, whose image is
-// at most half as large.
+// packed rows, read bit by bit, meet at 3 (2 bits) and 4.  From 160 x 160 on it is one
+// MCS more (191, S = 5, n = 3 38.5, 39.7).  Up to 128 x 128 n = 1 gains (L = 100 37.3,
+// 24.9).  Every other lattice that fits runs on macros, whose image is at most half as
+// large.
 bool resident_on_macros(const LatticeDesc& d, uint64_t n_mcs) {
   if (!slot_axis_ok(d.ax) || !slot_axis_ok(d.ay)) return false;
   const int planes = patch_planes(d);
   if (resident_layout(d, planes).bytes > kResPatchBytes) return false;
-  return (int64_t)d.L * d.H <= 16384 || n_mcs >= (uint64_t)(planes + (d.bits == 8 ? 1 : 2));
+  const int64_t sites = (int64_t)d.L * d.H;
+  return sites <= 16384 || n_mcs >= (uint64_t)(planes + (d.bits == 8 && sites < 25600 ? 1 : 2));
 }
 
 cudaError_t launch_resident(const PersistentArgs& a, cudaStream_t stream) {

@@ -102,9 +102,9 @@ def test_few_exchanges_move_the_line():
         g.close()
 
 
-@pytest.mark.parametrize("L,H,S,kw,line", [(128, 127, 3, {}, 1), (130, 129, 3, {}, 2), (191, 160, 5, {}, 3),
+@pytest.mark.parametrize("L,H,S,kw,line", [(128, 127, 3, {}, 1), (130, 129, 3, {}, 2), (150, 151, 5, {}, 3), (191, 160, 5, {}, 4),
                                            (160, 150, 3, dict(bits_per_site=2), 3), (160, 150, 5, dict(bits_per_site=4), 4),
-                                           (300, 270, 3, dict(persistent=4, reflecting_boundary=True), 2)])
+                                           (300, 270, 3, dict(persistent=4, reflecting_boundary=True), 3)])
 def test_resident_launches(L, H, S, kw, line):
     """The same line for whole-lattice residency, launch by launch."""
     D = O.circulant(S, (1,) if S == 3 else (1, 2))
